@@ -605,7 +605,7 @@ k_l2rev_e(const __grid_constant__ LagMaps m_, StepArgs a_) {
             for (int c = 0; c < 2; ++c) {
               const int xc = x + c;
               if ((c == 0 ? xyin0 : xyin1) && xc >= a.dlo[0] && xc < a.dhi[0]) {
-                const float s = lex[c] * c0[c] + ley[c] * c1[c] + lez[c] * c2[c];
+                const float s = grad_term(lex[c], ley[c], lez[c], c0[c], c1[c], c2[c]);
                 const long long qd =
                     ((long long)(k - a.dlo[2]) * dY + (y - a.dlo[1])) * dX + (xc - a.dlo[0]);
                 // one owner per cell: a fire-and-forget reduction in L2 adds
@@ -625,23 +625,23 @@ k_l2rev_e(const __grid_constant__ LagMaps m_, StepArgs a_) {
         float o6[2], o11[2], o7[2], o8[2], o9[2], o10[2];
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          const float wx = cbv[c] * lex[c], wy = cbv[c] * ley[c], wz = cbv[c] * lez[c];
+          const float wx = __fmul_rn(cbv[c], lex[c]), wy = __fmul_rn(cbv[c], ley[c]), wz = __fmul_rn(cbv[c], lez[c]);
           o6[c] = wx; o11[c] = -wz; o7[c] = -wx; o8[c] = wy; o9[c] = -wy; o10[c] = wz;
         }
         float n6[2], n11[2];
         {
           const float2 cy2 = ld2(CBb, hb + B::W);
           const float2 ly = ld2(LEb, hb + B::W), lz = ld2(LEb + 2 * B::P, hb + B::W);
-          n6[0] = cy2.x * ly.x;
-          n6[1] = cy2.y * ly.y;
-          n11[0] = -cy2.x * lz.x;
-          n11[1] = -cy2.y * lz.y;
+          n6[0] = __fmul_rn(cy2.x, ly.x);
+          n6[1] = __fmul_rn(cy2.y, ly.y);
+          n11[0] = __fmul_rn(-cy2.x, lz.x);
+          n11[1] = __fmul_rn(-cy2.y, lz.y);
         }
         float n9x, n10x;   // +x terms of cell 1 (from x + 2)
         {
           const float c2 = CBb[hb + 2];
-          n9x = -c2 * LEb[B::P + hb + 2];
-          n10x = c2 * LEb[2 * B::P + hb + 2];
+          n9x = __fmul_rn(-c2, LEb[B::P + hb + 2]);
+          n10x = __fmul_rn(c2, LEb[2 * B::P + hb + 2]);
         }
         if (y + 1 >= g.ny) {
           n6[0] = 0.f; n6[1] = 0.f; n11[0] = 0.f; n11[1] = 0.f;
@@ -745,10 +745,10 @@ k_l2rev_e(const __grid_constant__ LagMaps m_, StepArgs a_) {
         float n7[2] = {0.f, 0.f}, n8[2] = {0.f, 0.f};
         if (p < g.nz) {
           const float2 c2 = ld2(CBb, hb), lx = ld2(LEb, hb), ly = ld2(LEb + B::P, hb);
-          n7[0] = -c2.x * lx.x;
-          n7[1] = -c2.y * lx.y;
-          n8[0] = c2.x * ly.x;
-          n8[1] = c2.y * ly.y;
+          n7[0] = __fmul_rn(-c2.x, lx.x);
+          n7[1] = __fmul_rn(-c2.y, lx.y);
+          n8[0] = __fmul_rn(c2.x, ly.x);
+          n8[1] = __fmul_rn(c2.y, ly.y);
           if (in_slab(p, g.nz, g.P)) {
             const float* P = reinterpret_cast<const float*>(st + Y::PZ);
             const float b1 = prof(g, 2, PR_BE, p), a1 = prof(g, 2, PR_AE, p), k1v = prof(g, 2, PR_KE, p);
@@ -901,20 +901,20 @@ k_l2rev_h(const __grid_constant__ LagMaps m_, StepArgs a_) {
         float o0[2], o1[2], o2[2], o3[2], o4[2], o5[2];
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          o0[c] = -S_ * lhx[c];
-          o5[c] = S_ * lhz[c];
-          o1[c] = S_ * lhx[c];
-          o2[c] = -S_ * lhy[c];
-          o3[c] = S_ * lhy[c];
-          o4[c] = -S_ * lhz[c];
+          o0[c] = __fmul_rn(-S_, lhx[c]);
+          o5[c] = __fmul_rn(S_, lhz[c]);
+          o1[c] = __fmul_rn(S_, lhx[c]);
+          o2[c] = __fmul_rn(-S_, lhy[c]);
+          o3[c] = __fmul_rn(S_, lhy[c]);
+          o4[c] = __fmul_rn(-S_, lhz[c]);
         }
         float m0[2], m5[2];
         {
           const float2 lxy = ld2(LHb, lb - B::W), lzy = ld2(LHb + 2 * B::P, lb - B::W);   // -y
-          m0[0] = -S_ * lxy.x; m0[1] = -S_ * lxy.y;
-          m5[0] = S_ * lzy.x;  m5[1] = S_ * lzy.y;
+          m0[0] = __fmul_rn(-S_, lxy.x); m0[1] = __fmul_rn(-S_, lxy.y);
+          m5[0] = __fmul_rn(S_, lzy.x);  m5[1] = __fmul_rn(S_, lzy.y);
         }
-        float m3x = S_ * LHb[B::P + lb - 1], m4x = -S_ * LHb[2 * B::P + lb - 1];   // -x of cell 0
+        float m3x = __fmul_rn(S_, LHb[B::P + lb - 1]), m4x = __fmul_rn(-S_, LHb[2 * B::P + lb - 1]);   // -x of cell 0
         if (y == 0) { m0[0] = 0.f; m0[1] = 0.f; m5[0] = 0.f; m5[1] = 0.f; }
         if (x == 0) { m3x = 0.f; m4x = 0.f; }
         if (sy || sym) {
@@ -1002,8 +1002,8 @@ k_l2rev_h(const __grid_constant__ LagMaps m_, StepArgs a_) {
         float m1n[2] = {0.f, 0.f}, m2n[2] = {0.f, 0.f};
         if (p >= 0) {
           const float2 lx2 = ld2(LHb, lb), ly2 = ld2(LHb + B::P, lb);
-          m1n[0] = S_ * lx2.x; m1n[1] = S_ * lx2.y;
-          m2n[0] = -S_ * ly2.x; m2n[1] = -S_ * ly2.y;
+          m1n[0] = __fmul_rn(S_, lx2.x); m1n[1] = __fmul_rn(S_, lx2.y);
+          m2n[0] = __fmul_rn(-S_, ly2.x); m2n[1] = __fmul_rn(-S_, ly2.y);
           if (in_slab(p, g.nz, g.P)) {
             const float* P = reinterpret_cast<const float*>(st + Y::PZ);
             const float b1 = prof(g, 2, PR_BH, p), a1 = prof(g, 2, PR_AH, p), k1v = prof(g, 2, PR_KH, p);

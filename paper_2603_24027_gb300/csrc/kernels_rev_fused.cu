@@ -33,8 +33,7 @@
 // tile's pairs of cells; a fifth computes the halo (a row of 16 pairs and a
 // column of TY cells).  The primal half-steps repeat the forward's rounded
 // operations exactly, so the primal fields are bit-identical to the split
-// kernels'; the adjoint sums are left to the compiler's contraction, as in
-// the split kernels.
+// kernels', and so are the adjoint's (explicitly rounded products and sums).
 #include <cudaTypedefs.h>
 
 #include "lag_common.cuh"
@@ -246,7 +245,8 @@ k_rev_primal(const __grid_constant__ RevMaps m, StepArgs a) {
               const int xc = x + c;
               if ((c == 0 ? i0 : i1) && xc >= a.dlo[0] && xc < a.dhi[0]) {
                 const long long qc = q + c;
-                const float s = a.L[qc] * c0[c] + a.L[nc + qc] * c1[c] + a.L[2 * nc + qc] * c2[c];
+                const float s =
+                        grad_term(a.L[qc], a.L[nc + qc], a.L[2 * nc + qc], c0[c], c1[c], c2[c]);
                 const long long qd =
                     ((long long)(p - a.dlo[2]) * dY + (y - a.dlo[1])) * dX + (xc - a.dlo[0]);
 #ifdef FDTD_BOUNDS_CHECK
@@ -462,22 +462,22 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
           const float cbv[2] = {cb2.x, cb2.y};
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
-            const float wx = cbv[c] * own_le[0][c], wy = cbv[c] * own_le[1][c],
-                        wz = cbv[c] * own_le[2][c];
+            const float wx = __fmul_rn(cbv[c], own_le[0][c]), wy = __fmul_rn(cbv[c], own_le[1][c]),
+                        wz = __fmul_rn(cbv[c], own_le[2][c]);
             o6[c] = wx; o11[c] = -wz; o7[c] = -wx; o8[c] = wy; o9[c] = -wy; o10[c] = wz;
           }
           if (y + 1 < g.ny) {
             const float2 cy2 = ld2(CBb, wb + Y::WW);
             const float2 ly = ld2(LEb, wb + Y::WW), lz = ld2(LEb + 2 * Y::WP, wb + Y::WW);
-            n6[0] = cy2.x * ly.x;
-            n6[1] = cy2.y * ly.y;
-            n11[0] = -cy2.x * lz.x;
-            n11[1] = -cy2.y * lz.y;
+            n6[0] = __fmul_rn(cy2.x, ly.x);
+            n6[1] = __fmul_rn(cy2.y, ly.y);
+            n11[0] = __fmul_rn(-cy2.x, lz.x);
+            n11[1] = __fmul_rn(-cy2.y, lz.y);
           }
           if (x + 2 < g.nx) {
             const float c2 = CBb[wb + 2];
-            n9x = -c2 * LEb[Y::WP + wb + 2];
-            n10x = c2 * LEb[2 * Y::WP + wb + 2];
+            n9x = __fmul_rn(-c2, LEb[Y::WP + wb + 2]);
+            n10x = __fmul_rn(c2, LEb[2 * Y::WP + wb + 2]);
           }
         }
         if (PXY) {
@@ -597,10 +597,10 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
         float n7[2] = {0.f, 0.f}, n8[2] = {0.f, 0.f};
         if (inz(p)) {
           const float2 c2 = ld2(CBb, wb), lx = ld2(LEb, wb), ly = ld2(LEb + Y::WP, wb);
-          n7[0] = -c2.x * lx.x;
-          n7[1] = -c2.y * lx.y;
-          n8[0] = c2.x * ly.x;
-          n8[1] = c2.y * ly.y;
+          n7[0] = __fmul_rn(-c2.x, lx.x);
+          n7[1] = __fmul_rn(-c2.y, lx.y);
+          n8[0] = __fmul_rn(c2.x, ly.x);
+          n8[1] = __fmul_rn(c2.y, ly.y);
           if (zs) {
             const float* P = reinterpret_cast<const float*>(st + Y::PEZ);
             const float b1 = prof(g, 2, PR_BE, p), a1 = prof(g, 2, PR_AE, p), k1v = prof(g, 2, PR_KE, p);
@@ -638,21 +638,21 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
           const float lhx[2] = {lx2.x, lx2.y}, lhy[2] = {ly2.x, ly2.y}, lhz[2] = {lz2.x, lz2.y};
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
-            o0[c] = -S_ * lhx[c];
-            o5[c] = S_ * lhz[c];
-            o1[c] = S_ * lhx[c];
-            o2[c] = -S_ * lhy[c];
-            o3[c] = S_ * lhy[c];
-            o4[c] = -S_ * lhz[c];
+            o0[c] = __fmul_rn(-S_, lhx[c]);
+            o5[c] = __fmul_rn(S_, lhz[c]);
+            o1[c] = __fmul_rn(S_, lhx[c]);
+            o2[c] = __fmul_rn(-S_, lhy[c]);
+            o3[c] = __fmul_rn(S_, lhy[c]);
+            o4[c] = __fmul_rn(-S_, lhz[c]);
           }
         }
         float m0[2], m5[2];
         {
           const float2 lxy = ld2(SL, lb - Y::HW), lzy = ld2(SL + 2 * Y::HP, lb - Y::HW);   // -y
-          m0[0] = -S_ * lxy.x; m0[1] = -S_ * lxy.y;
-          m5[0] = S_ * lzy.x;  m5[1] = S_ * lzy.y;
+          m0[0] = __fmul_rn(-S_, lxy.x); m0[1] = __fmul_rn(-S_, lxy.y);
+          m5[0] = __fmul_rn(S_, lzy.x);  m5[1] = __fmul_rn(S_, lzy.y);
         }
-        float m3x = S_ * SL[Y::HP + lb - 1], m4x = -S_ * SL[2 * Y::HP + lb - 1];   // -x of cell 0
+        float m3x = __fmul_rn(S_, SL[Y::HP + lb - 1]), m4x = __fmul_rn(-S_, SL[2 * Y::HP + lb - 1]);   // -x of cell 0
         if (y == 0) { m0[0] = 0.f; m0[1] = 0.f; m5[0] = 0.f; m5[1] = 0.f; }
         if (x == 0) { m3x = 0.f; m4x = 0.f; }
         const int pm = p - 1;
@@ -752,8 +752,8 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
         if (pm >= 0) {
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
-            m1n[c] = S_ * fx[c];
-            m2n[c] = -S_ * fy[c];
+            m1n[c] = __fmul_rn(S_, fx[c]);
+            m2n[c] = __fmul_rn(-S_, fy[c]);
           }
           if (PZ && in_slab(pm, g.nz, g.P)) {
             const float* P = reinterpret_cast<const float*>(st + Y::PHZ);

@@ -212,8 +212,8 @@ __device__ __forceinline__ void restore_seed_body(float* __restrict__ F, float* 
       const int s = ip.slot[fld][m];
       if (s >= 0) {
         float x = Code<DT>::dec(tp[(long long)s * stride]);
-        if (DT >= 2) x = x * __ldg(scales + s * 6 + f);
-        val += ip.w[fld][m] * x;
+        if (DT >= 2) x = __fmul_rn(x, __ldg(scales + s * 6 + f));
+        val = __fmaf_rn(ip.w[fld][m], x, val);
       }
     }
     int comp;

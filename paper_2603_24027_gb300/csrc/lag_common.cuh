@@ -141,12 +141,20 @@ __device__ __forceinline__ float cpml(float d, float psi_old, float b, float a, 
   return __fmaf_rn(kv, d, t);
 }
 
-// Adjoint of the recursion: returns the curl term with the CPML response;
+// Adjoint of the recursion: returns the curl term with the CPML response.  The
+// adjoint's products and sums are rounded explicitly, in the same order in every
+// kernel, so that its fields and the gradient do not depend on which kernels run;
 // the adjoint auxiliary for the next (earlier) step goes to *out.
 __device__ __forceinline__ float adj(float v, float lpsi, float b, float a, float kv, float* out) {
   const float mu = lpsi + v;
   *out = b * mu;
-  return kv * v + a * mu;
+  return __fmaf_rn(a, mu, __fmul_rn(kv, v));
+}
+
+// lam_E . (curl Ht - J): one cell's part of dL/dcb.
+__device__ __forceinline__ float grad_term(float lx, float ly, float lz, float c0, float c1,
+                                           float c2) {
+  return __fmaf_rn(lz, c2, __fmaf_rn(ly, c1, __fmul_rn(lx, c0)));
 }
 
 // Programmatic dependent launch: wait until the previous kernel in the stream

@@ -25,6 +25,9 @@ __device__ __forceinline__ long long face_value_cell(const Geo& g, const FaceDes
   return cell_on_plane(g, fd.axis, fd.layer, g.P + u, g.P + v);
 }
 
+// An objective seed: *l += s v, rounded once.
+__device__ __forceinline__ void add_seed(float* l, float s, float v) { *l = __fmaf_rn(s, v, *l); }
+
 // Detector blocks of the restore launch: block b (of det_blocks per
 // detector) adds the objective seeds on the detector planes: seeds[0] *
 // dl_n/d(E^{n+1}, Ht^{n+1/2}) for the detector, seeds[1] * dm_n/d(...) for the
@@ -43,15 +46,15 @@ __device__ __forceinline__ void seed_detectors(float* __restrict__ F, float* __r
   const int v = r / du, e = r - v * du;
   const long long q = cell_on_plane(g, d.axis, d.index, d.u0 + e, d.v0 + v);
   if (d.kind == 1) {
-    for (int c = 0; c < 3; ++c) L[c * g.nc + q] += s * (2.0f * F[c * g.nc + q]);
+    for (int c = 0; c < 3; ++c) add_seed(&L[c * g.nc + q], s, 2.0f * F[c * g.nc + q]);
   } else {
     const int bb = (d.axis + 1) % 3, c = (d.axis + 2) % 3;
     const float Eb = F[bb * g.nc + q], Ec = F[c * g.nc + q];
     const float Hb = F[(3 + bb) * g.nc + q], Hc = F[(3 + c) * g.nc + q];
-    L[bb * g.nc + q] += s * Hc;
-    L[c * g.nc + q] -= s * Hb;
-    L[(3 + c) * g.nc + q] += s * Eb;
-    L[(3 + bb) * g.nc + q] -= s * Ec;
+    add_seed(&L[bb * g.nc + q], s, Hc);
+    add_seed(&L[c * g.nc + q], -s, Hb);
+    add_seed(&L[(3 + c) * g.nc + q], s, Eb);
+    add_seed(&L[(3 + bb) * g.nc + q], -s, Ec);
   }
 }
 
