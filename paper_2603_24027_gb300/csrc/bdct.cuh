@@ -41,6 +41,45 @@ BdctLayout bdct_layout(const Faces& fc, int K);
 // Upload the basis table to the device once per device (host-synchronous;
 // call outside stream capture).
 cudaError_t bdct_ensure_basis();
+// The uploaded table of the current device, or NULL before its upload (no
+// runtime call a stream capture forbids).
+const float* bdct_basis_device();
+
+// Value of cell t (y * 8 + x) of a block from its K codes and scale.
+__device__ __forceinline__ float bdct_decode_cell(const signed char* __restrict__ codes, float s,
+                                                  int K, int t, const float* __restrict__ beta) {
+  float acc = 0.f;
+  for (int i = 0; i < K; ++i)
+    acc = __fmaf_rn((float)codes[i], __ldg(beta + i * 64 + t), acc);
+  return __fmul_rn(acc, s);
+}
+
+// Value rr of face f restored from the samples of ip.
+__device__ __forceinline__ float bdct_restored(const BdctLayout& bl, const FaceDesc& fd, int f,
+                                               int rr, const unsigned char* __restrict__ tape,
+                                               long long stride, const Interp& ip,
+                                               const float* __restrict__ beta) {
+  const int row = rr / fd.nu, u = rr - row * fd.nu;
+  const int comp_t = row >= fd.nv, v = row - comp_t * fd.nv;
+  const int bu = u >> 3, bv = v >> 3;
+  const int b = bl.bstart[f] + comp_t * bl.nbu[f] * bl.nbv[f] + bv * bl.nbu[f] + bu;
+  const int t = (v & 7) * 8 + (u & 7);
+  const int fld = f & 1;  // 0: Ht on low faces, 1: E on high faces
+  float val = 0.f;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const int s = ip.slot[fld][m];
+    if (s >= 0) {
+      const unsigned char* smp = tape + (long long)s * stride;
+      const float sc = __ldg(reinterpret_cast<const float*>(smp + bl.code_bytes) + b);
+      const float x =
+          bdct_decode_cell(reinterpret_cast<const signed char*>(smp) + (long long)b * bl.K, sc,
+                           bl.K, t, beta);
+      val = __fmaf_rn(ip.w[fld][m], x, val);
+    }
+  }
+  return val;
+}
 
 cudaError_t launch_record_bdct(const float* FH, const float* FE, Geo g, const Faces& fc,
                                const BdctLayout& bl, void* tape_sample, cudaStream_t s);

@@ -21,6 +21,7 @@
 
 #include "../../include/fdtd.h"
 #include "bdct.cuh"
+#include "direct.cuh"
 #include "fdtd_internal.cuh"
 
 using namespace fdtd;
@@ -497,10 +498,34 @@ static bool two_step_forward(const fdtd_handle* h) {
   return R.ix1 > R.ix0 && 2 * cpml <= all;
 }
 
+// Small grids run the direct half-steps (kernels_direct.cu) unless an option
+// names another form or shape.  The lines lie where they stop being faster
+// than the split staged ones (us per step, direct against split): forward
+// 5.2 / 26.7 at 0.11 M cells, 16.1 / 30.5 at 1.2 M, 23.6 / 35.1 at 1.8 M, 35.3 /
+// 38.5 at 2.6 M, 50.5 / 50.1 at 3.2 M, 63.5 / 60.1 at 4 M; reverse 6.9 / 30.6 at
+// 0.11 M, 27.6 / 39.0 at 1.2 M, 53.0 / 57.2 at 1.8 M, 78 / 73 at 2.6 M, 120 / 104 at
+// 4 M (beyond the L2 cache its re-read neighbour planes come from HBM).
+static const long long kDirectForwardCells = 3000000, kDirectReverseCells = 2000000;
+static bool direct_shape(const fdtd_handle* h) {
+  return h->opt_kernel == 5 && h->opt_tile_y == 8 && h->opt_tile_x == 32 && h->opt_stages == 2 &&
+         h->opt_zchunk == 8 && h->opt_zchunk_fwd == -1 && h->opt_zgroups <= 1 && !h->opt_pdl &&
+         !h->opt_prefetch;
+}
+static Geo geo_of(const fdtd_handle* h);
+static bool direct_forward(const fdtd_handle* h) {
+  return direct_shape(h) && direct_fits(geo_of(h)) && h->opt_forward == 0 &&
+         (long long)h->nx * h->ny * h->nz <= kDirectForwardCells;
+}
+static bool direct_reverse(const fdtd_handle* h) {
+  return direct_shape(h) && direct_fits(geo_of(h)) && h->opt_reverse == 0 &&
+         (long long)h->nx * h->ny * h->nz <= kDirectReverseCells;
+}
+
 // The field buffer holding the state after a forward: the fused step flips
 // the pair every step, the two-step pass every pair of steps (and its split
 // first step, for an odd count, once).
 static int forward_end_buf(const fdtd_handle* h) {
+  if (direct_forward(h)) return 0;
   if (two_step_forward(h)) return ((h->N + 1) / 2) & 1;
   return fused_forward(h) ? (h->N & 1) : 0;
 }
@@ -1055,6 +1080,23 @@ static StepArgs step_args(const fdtd_handle* h, const Layout& L) {
   return a;
 }
 
+// What the direct half-steps take from the step arguments.
+static DirectArgs direct_args(const fdtd_handle* h, const Layout& L, const StepArgs& a) {
+  DirectArgs d;
+  memset(&d, 0, sizeof d);
+  d.g = a.g;
+  d.cb = a.cb;
+  d.pl = a.pl;
+  d.gacc = a.gacc;
+  for (int i = 0; i < 3; ++i) { d.dlo[i] = a.dlo[i]; d.dhi[i] = a.dhi[i]; }
+  d.src = a.src;
+  d.det = a.det;
+  d.xq = a.xq; d.xs = a.xs; d.xi = a.xi;
+  d.fc = h->faces;
+  d.err = a.err;
+  return d;
+}
+
 // Sampled kernel timing: event pairs recorded on h->stream around every
 // opt_sample-th launch of a kernel kind (external event nodes when captured).
 // Sampled kernel timing.  A CUDA event pair around a single launch inside the
@@ -1291,6 +1333,48 @@ static cudaError_t enqueue_forward(fdtd_handle* h, const fdtd_record_cfg* rec, i
   if (det2.kind && (e = cudaMemsetAsync(h->ws + L.obj2, 0, h->N * sizeof(double), h->stream)))
     return e;
   Sampler smp(h, 0);
+  if (direct_forward(h)) {
+    // two launches per step; an unscaled record rides in them unless kernel
+    // timing is being sampled (which times one kind per launch)
+    DirectArgs d = direct_args(h, L, a);
+    const bool fold = h->opt_sample == 0;
+    const bool ride = fold && !bdct && !(rec->scaled && rec->dtype >= 2);
+    d.psiA = a.psiA;
+    d.F = a.F;
+    d.tdtype = rec->dtype;
+    if (fold) d.det2 = det2;
+    for (int n = 0; n < h->N; ++n) {
+      const bool rec_now = n >= r && (n - r) % rec->k == 0;
+      const int j = rec_now ? (n - r) / rec->k : 0;
+      d.jn = h->wave[n];
+      d.obj = (double*)(h->ws + L.obj) + n;
+      d.obj2 = (double*)(h->ws + L.obj2) + n;
+      d.tmode = rec_now && ride;
+      d.tape = tape + (size_t)j * L.stride * eb;
+      d.scale_slot = scales + (size_t)j * 6;
+      if ((e = smp.before(FDTD_K_FWD_H))) return e;
+      if ((e = launch_direct(0, d, h->stream))) return e;
+      if ((e = smp.after(FDTD_K_FWD_H))) return e;
+      if (rec_now && !ride) {
+        if ((e = smp.before(FDTD_K_RECORD))) return e;
+        if ((e = record(a.F, a.F, j))) return e;
+        if ((e = smp.after(FDTD_K_RECORD))) return e;
+        ++nl;
+      }
+      if ((e = smp.before(FDTD_K_FWD_E))) return e;
+      if ((e = launch_direct(1, d, h->stream))) return e;
+      if ((e = smp.after(FDTD_K_FWD_E))) return e;
+      nl += 2;
+      if (det2.kind && !fold) {
+        if ((e = smp.before(FDTD_K_MONITOR))) return e;
+        if ((e = launch_monitor(a.F, a.g, det2, d.obj2, h->stream))) return e;
+        if ((e = smp.after(FDTD_K_MONITOR))) return e;
+        ++nl;
+      }
+    }
+    *launches = nl;
+    return cudaSuccess;
+  }
   if (two_step_forward(h)) {
     // two steps per pass: steps n, n + 1 of the deep units in one launch on
     // the main stream (buffer cur -> cur ^ 1, the intermediate level's frame
@@ -1541,7 +1625,8 @@ static cudaError_t enqueue_backward(fdtd_handle* h, const fdtd_record_cfg* rec, 
   int nl = 0;
   // the adjoint starts at zero in the buffer the first step reads: the fused
   // reverse step starts in the forward's buffer, the split phases work in 0
-  const int lam0 = fused_reverse(h) ? h->fwd_buf : 0;
+  const bool direct = direct_reverse(h), fused = !direct && fused_reverse(h);
+  const int lam0 = fused ? h->fwd_buf : 0;
   if ((e = cudaMemsetAsync(h->ws + L.L[lam0], 0, nc6, h->stream))) return e;
   if ((e = cudaMemsetAsync(h->ws + L.psiL[0], 0, psb, h->stream))) return e;
   if ((e = cudaMemsetAsync(h->ws + L.psiL[1], 0, psb, h->stream))) return e;
@@ -1556,8 +1641,7 @@ static cudaError_t enqueue_backward(fdtd_handle* h, const fdtd_record_cfg* rec, 
   Det det = a.det;
   const Det det2 = det2_of(h);
   int cur = h->fwd_buf;   // the forward's final state
-  const bool fused = fused_reverse(h);
-  const bool rpair = h->opt_kernel == 5 && !fused;
+  const bool rpair = h->opt_kernel == 5 && !fused && !direct;
   LagMaps lrmaps[2];
   for (int b = 0; b < 2; ++b)
     if (rpair && (e = encode_lag_maps(a.F, a.L, (const float*)(h->ws + L.cb),
@@ -1581,6 +1665,58 @@ static cudaError_t enqueue_backward(fdtd_handle* h, const fdtd_record_cfg* rec, 
   const BdctLayout bl =
       rec->dtype == kTapeBdct ? bdct_layout(h->faces, bdct_coeffs(rec)) : BdctLayout{};
   Sampler smp(h, 1);
+  if (direct) {
+    // two launches per step: the tape's restore and the objective seeds of a
+    // step ride in the launches of the step before it in reverse order, after
+    // one restore launch that starts the loop (every step has its own while
+    // kernel timing is being sampled)
+    DirectArgs d = direct_args(h, L, a);
+    const bool bd = rec->dtype == kTapeBdct;
+    d.beta = bd ? bdct_basis_device() : nullptr;
+    d.bl = bl;
+    const bool ride = h->opt_sample == 0 && (!bd || d.beta);
+    d.F = a.F;
+    d.L = a.L;
+    d.det2 = det2;
+    d.seeds = (const double*)(h->ws + L.seeds);
+    d.tdtype = rec->dtype;
+    d.tape = h->ws + L.tape;
+    d.stride = L.stride;
+    d.scales = (const float*)(h->ws + L.scales);
+    for (int n = h->N - 1; n >= 0; --n) {
+      Interp ip;
+      interp_weights(h, rec, n, 0, ip.slot[0], ip.w[0]);
+      interp_weights(h, rec, n, 1, ip.slot[1], ip.w[1]);
+      const bool first = n == h->N - 1;
+      if (first || !ride) {
+        if ((e = smp.before(FDTD_K_RESTORE))) return e;
+        if ((e = bd ? launch_restore_seed_bdct(a.F, a.L, a.g, h->faces, bl, h->ws + L.tape,
+                                               L.stride, ip, det, det2, d.seeds, h->stream)
+                    : launch_restore_seed(rec->dtype, a.F, a.L, a.g, h->faces, h->ws + L.tape,
+                                          L.stride, d.scales, ip, det, det2, d.seeds, h->stream)))
+          return e;
+        if ((e = smp.after(FDTD_K_RESTORE))) return e;
+        ++nl;
+      }
+      d.jn = h->wave[n];
+      d.psiA = (float*)(h->ws + L.psiL[cur]);
+      d.psiB = (float*)(h->ws + L.psiL[cur ^ 1]);
+      d.ip = ip;
+      d.tmode = d.seeded = ride && !first;
+      if ((e = smp.before(FDTD_K_REV_E))) return e;
+      if ((e = launch_direct(2, d, h->stream))) return e;
+      if ((e = smp.after(FDTD_K_REV_E))) return e;
+      d.tmode = d.seeded = ride && n > 0;
+      if (n > 0) interp_weights(h, rec, n - 1, 0, d.ip.slot[0], d.ip.w[0]);
+      if ((e = smp.before(FDTD_K_REV_H))) return e;
+      if ((e = launch_direct(3, d, h->stream))) return e;
+      if ((e = smp.after(FDTD_K_REV_H))) return e;
+      cur ^= 1;
+      nl += 2;
+    }
+    *launches = nl;
+    return cudaSuccess;
+  }
   ZGroups zg(h, rpair, 1, a);
   if (zg.active()) smp.m = 0;   // launches of a phase overlap: no per-kind intervals
   for (int n = h->N - 1; n >= 0; --n) {
@@ -1874,7 +2010,7 @@ static int backward_async(fdtd_handle* h, double seed, double seed2) {
   h->have_forward = false;
   // the fused reverse step leaves the reconstructed fields in the buffer of
   // the last step's output
-  if (fused_reverse(h)) h->fwd_buf ^= h->N & 1;
+  if (!direct_reverse(h) && fused_reverse(h)) h->fwd_buf ^= h->N & 1;
   return FDTD_OK;
 }
 

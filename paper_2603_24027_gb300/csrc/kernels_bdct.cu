@@ -72,23 +72,33 @@ BdctLayout bdct_layout(const Faces& fc, int K) {
   return bl;
 }
 
+static std::mutex g_basis_mu;
+static const float* g_basis_ptr[64];   // the uploaded table of each device
+
 cudaError_t bdct_ensure_basis() {
-  static std::mutex mu;
-  static bool done[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::lock_guard<std::mutex> lock(mu);
-  if (done[dev]) return cudaSuccess;
+  std::lock_guard<std::mutex> lock(g_basis_mu);
+  if (g_basis_ptr[dev]) return cudaSuccess;
+  void* p = nullptr;
+  if ((e = cudaGetSymbolAddress(&p, g_bdct_beta))) return e;
   float beta[64 * 64], beta_t[64 * 64];
   bdct_basis_host(beta);
   for (int i = 0; i < 64; ++i)
     for (int t = 0; t < 64; ++t) beta_t[t * 64 + i] = beta[i * 64 + t];
   if ((e = cudaMemcpyToSymbol(g_bdct_beta, beta, sizeof beta))) return e;
   if ((e = cudaMemcpyToSymbol(g_bdct_beta_t, beta_t, sizeof beta_t))) return e;
-  done[dev] = true;
+  g_basis_ptr[dev] = (const float*)p;
   return cudaSuccess;
+}
+
+const float* bdct_basis_device() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+  std::lock_guard<std::mutex> lock(g_basis_mu);
+  return g_basis_ptr[dev];
 }
 
 // ---------------------------------------------------------- device side ---
@@ -123,15 +133,6 @@ __device__ __forceinline__ void bdct_encode_block_warp(const float* X, int K, in
     }
   }
   if (lane == 0) *scale = s;
-}
-
-// Value of cell t (y * 8 + x) of a block from its K codes and scale.
-__device__ __forceinline__ float bdct_decode_cell(const signed char* __restrict__ codes, float s,
-                                                  int K, int t) {
-  float acc = 0.f;
-  for (int i = 0; i < K; ++i)
-    acc = __fmaf_rn((float)codes[i], __ldg(g_bdct_beta + i * 64 + t), acc);
-  return __fmul_rn(acc, s);
 }
 
 static constexpr int BDCT_WARPS = BDCT_THREADS / 32;
@@ -194,25 +195,7 @@ __global__ void __launch_bounds__(BDCT_THREADS) k_restore_seed_bdct(
     for (int t = 1; t < 6; ++t) f += r >= fc.start[t];
     const FaceDesc& fd = fc.f[f];
     const int rr = r - fc.start[f];
-    const int row = rr / fd.nu, u = rr - row * fd.nu;
-    const int comp_t = row >= fd.nv, v = row - comp_t * fd.nv;
-    const int bu = u >> 3, bv = v >> 3;
-    const int b = bl.bstart[f] + comp_t * bl.nbu[f] * bl.nbv[f] + bv * bl.nbu[f] + bu;
-    const int t = (v & 7) * 8 + (u & 7);
-    const int fld = f & 1;  // 0: Ht on low faces, 1: E on high faces
-    float val = 0.f;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int s = ip.slot[fld][m];
-      if (s >= 0) {
-        const unsigned char* smp = tape + (long long)s * stride;
-        const float sc = __ldg(reinterpret_cast<const float*>(smp + bl.code_bytes) + b);
-        const float x =
-            bdct_decode_cell(reinterpret_cast<const signed char*>(smp) + (long long)b * bl.K, sc,
-                             bl.K, t);
-        val += ip.w[fld][m] * x;
-      }
-    }
+    const float val = bdct_restored(bl, fd, f, rr, tape, stride, ip, g_bdct_beta);
     int comp;
     const long long q = face_value_cell(g, fd, rr, &comp);
     F[comp * g.nc + q] = val;
@@ -267,7 +250,8 @@ __global__ void __launch_bounds__(BDCT_THREADS) k_bdct_decode(const signed char*
   const int v = (int)(r / nu), u = (int)(r - (long long)v * nu);
   const int nbu = (nu + 7) / 8;
   const int b = (v >> 3) * nbu + (u >> 3);
-  out[r] = bdct_decode_cell(codes + (long long)b * K, __ldg(scales + b), K, (v & 7) * 8 + (u & 7));
+  out[r] = bdct_decode_cell(codes + (long long)b * K, __ldg(scales + b), K, (v & 7) * 8 + (u & 7),
+                            g_bdct_beta);
 }
 
 cudaError_t launch_bdct_encode(const float* in, int nu, int nv, int K, signed char* codes,

@@ -1,0 +1,91 @@
+"""Direct half-steps of small grids (csrc/kernels_direct.cu) on the GPU.
+
+With default options a small grid runs the direct half-steps; asking for the
+split half-steps (FDTD_OPT_FORWARD = FDTD_OPT_REVERSE = 1) runs the staged
+kernels.  Both evaluate the same rounded operations, so the final fields, the
+tape, the reversed interior and the gradient must be equal bit for bit; the
+objectives' FP64 sums may differ in their order.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def F():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_2603_24027_gb300 import fdtd
+    return fdtd
+
+
+def _grid(name):
+    from paper_2603_24027_gb300 import inputs as I
+    if name == "min":         # a two-cell interior: one pair in an interior row
+        return I.fd_cube().replace(nx=6, ny=6, nz=6, eps=np.ones((6, 6, 6), np.float32),
+                                   design_lo=(2, 2, 2), design_hi=(4, 4, 4), src_pos=(2, 3, 2),
+                                   det_index=3, det_lo=(2, 2), det_hi=(4, 4))
+    if name == "thin":        # one-cell CPML, odd sizes, fewer cells than a CTA in a plane
+        return I.ragged_box(nx=13, ny=17, nz=15, P=1, n_steps=41)
+    if name == "odd":         # odd CPML: interior pairs cut in half on both sides
+        return I.ragged_box(nx=71, ny=33, nz=29, P=5, n_steps=60, det_kind=I.OBJ_E2_PLANE,
+                            src_kind=I.SRC_POINT)
+    if name == "compact":     # long enough for compact auxiliaries on every axis
+        return I.ragged_box(nx=150, ny=60, nz=40, P=7, n_steps=50)
+    return I.coupler_small(n_steps=70)   # two detectors
+
+
+def _run(F, w, rec, options):
+    sim = F.Simulation(w, device="cuda")
+    for k, v in options.items():
+        sim.set_option(k, v)
+    sim.ensure_workspace(rec).zero_()   # row and sample padding, which the saved state includes
+    sim.forward(torch.from_numpy(w.eps).cuda(), rec)
+    hist, obj = sim.objective_history(), sim.objectives()
+    fields, state = sim.read_fields().clone(), sim.save_state()
+    g = sim.backward(0.75, seed2=-0.5 if w.det2_kind else None).double().cpu().numpy()
+    return dict(hist=hist, obj=obj, fields=fields, state=state, grad=g, back=sim.read_fields(),
+                launches=sim.last_timing())
+
+
+@pytest.mark.parametrize("exact", [0, 22])
+@pytest.mark.parametrize("tape,k,interp", [("f32", 1, "linear"), ("bf16", 3, "cubic"),
+                                           ("e4m3", 4, "linear"), ("e5m2fnuz", 5, "cubic"),
+                                           ("bdct", 4, "cubic")])
+@pytest.mark.parametrize("name", ["min", "thin", "odd", "compact", "two"])
+def test_direct_half_steps_equal_the_staged_ones(F, name, tape, k, interp, exact):
+    from paper_2603_24027_gb300 import _capi as A
+    w = _grid(name)
+    rec = A.record_cfg(tape, k, interp)
+    ex = {A.OPT_EXACT_REVERSAL: exact}
+    a = _run(F, w, rec, ex)
+    b = _run(F, w, rec, {**ex, A.OPT_FORWARD: 1, A.OPT_REVERSE: 1})
+    # two launches a reverse step (and one that starts the loop)
+    assert a["launches"]["bwd_launches"] == 2 * w.n_steps + 1
+    assert torch.equal(a["fields"], b["fields"])
+    P = w.pml_thickness
+    core = (slice(None),) + tuple(slice(P, n - P) for n in (w.nz, w.ny, w.nx))
+    assert torch.equal(a["back"][core], b["back"][core])
+    # the saved state holds the tape
+    n = 8 * w.n_steps * 2
+    head = len(a["state"]) - n
+    skip = 128   # header: the second objective's sum
+    assert np.array_equal(a["state"][skip:head], b["state"][skip:head])
+    np.testing.assert_allclose(a["hist"], b["hist"], rtol=0, atol=1e-12 * np.abs(b["hist"]).max())
+    np.testing.assert_allclose(a["obj"], b["obj"], rtol=1e-11)
+    assert np.array_equal(a["grad"], b["grad"])
+
+
+def test_sampled_timing_of_a_small_grid_keeps_its_kinds(F):
+    """With kernel timing sampled, every kind has its own launch again; the results stay."""
+    from paper_2603_24027_gb300 import _capi as A
+    w = _grid("two")
+    rec = A.record_cfg("bf16", 2)
+    a = _run(F, w, rec, {})
+    b = _run(F, w, rec, {A.OPT_SAMPLE_EVERY: 3})
+    assert torch.equal(a["fields"], b["fields"])
+    assert a["launches"]["fwd_launches"] == 2 * w.n_steps
+    assert b["launches"]["fwd_launches"] == 3 * w.n_steps + (w.n_steps + 1) // 2
+    assert b["launches"]["bwd_launches"] == 3 * w.n_steps
