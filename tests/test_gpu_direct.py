@@ -34,7 +34,14 @@ def _grid(name):
                             src_kind=I.SRC_POINT)
     if name == "compact":     # long enough for compact auxiliaries on every axis
         return I.ragged_box(nx=150, ny=60, nz=40, P=7, n_steps=50)
-    return I.coupler_small(n_steps=70)   # two detectors
+    w = I.coupler_small(n_steps=70)   # two detectors
+    if name == "two":
+        return w
+    # crossing planes: cells that both detectors seed
+    P = w.pml_thickness
+    return w.replace(det_kind=I.OBJ_E2_PLANE, det_axis=0, det_index=P + 8, det_lo=(P, P),
+                     det_hi=(w.ny - P, w.nz - P), det2_kind=I.OBJ_POYNTING_PLANE, det2_axis=1,
+                     det2_index=w.ny - P - 1, det2_lo=(P, P), det2_hi=(w.nx - P, w.nz - P))
 
 
 def _run(F, w, rec, options):
@@ -54,7 +61,7 @@ def _run(F, w, rec, options):
 @pytest.mark.parametrize("tape,k,interp", [("f32", 1, "linear"), ("bf16", 3, "cubic"),
                                            ("e4m3", 4, "linear"), ("e5m2fnuz", 5, "cubic"),
                                            ("bdct", 4, "cubic")])
-@pytest.mark.parametrize("name", ["min", "thin", "odd", "compact", "two"])
+@pytest.mark.parametrize("name", ["min", "thin", "odd", "compact", "two", "cross"])
 def test_direct_half_steps_equal_the_staged_ones(F, name, tape, k, interp, exact):
     from paper_2603_24027_gb300 import _capi as A
     w = _grid(name)
@@ -89,3 +96,15 @@ def test_sampled_timing_of_a_small_grid_keeps_its_kinds(F):
     assert a["launches"]["fwd_launches"] == 2 * w.n_steps
     assert b["launches"]["fwd_launches"] == 3 * w.n_steps + (w.n_steps + 1) // 2
     assert b["launches"]["bwd_launches"] == 3 * w.n_steps
+
+
+@pytest.mark.parametrize("options", [{}, {"OPT_FORWARD": 1, "OPT_REVERSE": 1}])
+def test_detectors_that_share_cells(F, options):
+    """Both detectors' seeds arrive at the cells their planes share: the gradient of the
+    weighted sum against the FP64 oracle."""
+    from oracle import oracle as O
+    from paper_2603_24027_gb300 import _capi as A
+    w = _grid("cross")
+    r = _run(F, w, A.record_cfg("f32", 1), {getattr(A, k): v for k, v in options.items()})
+    _, _, g = O.gradient2(w, 0.75, -0.5)
+    assert np.linalg.norm(r["grad"] - g) <= 1e-4 * np.linalg.norm(g)
