@@ -34,6 +34,15 @@
 // column of TY cells).  The primal half-steps repeat the forward's rounded
 // operations exactly, so the primal fields are bit-identical to the split
 // kernels', and so are the adjoint's (explicitly rounded products and sums).
+//
+// What bounds them: DRAM for the launches together (600 x 600 x 300: 12.2 GB per
+// reverse step in 1974 us, 6.2 TB/s, 0.91 of the measured copy), and before
+// that the instructions per cell.  The primal units inside the interior carry no
+// predicate (FULL), the exchange between the two half-steps happens in the
+// staged box itself, one block barrier per plane is left in the primal and two
+// in the adjoint (three before), and stores address a plane's uniform base with a
+// 32-bit offset: 2071 -> 1974 us per reverse step (600 x 600 x 300), 671 -> 639
+// (411 x 389 x 203), 239 -> 218 (301 x 203 x 151).
 #include <cudaTypedefs.h>
 
 #include "lag_common.cuh"
@@ -47,8 +56,7 @@ namespace revf {
 // Shared memory of the primal kernel (byte offsets): S stages of an Ht box
 // (TW+8) x (TY+2) at (x0-4, y0-1) and E and cb boxes (TW+4) x (TY+1) at
 // (x0, y0); the stages' mbarriers right after them (where ring_init puts
-// them); then E^n of the plane on the tile and its +x / +y halo,
-// [3][TY+1][TW+4] at (x0, y0).
+// them).  E^n of a plane replaces E^{n+1} in its stage's E box.
 template <int TY, int S, int TW>
 struct PL {
   static constexpr int HW = TW + 8, HR = TY + 2, HP = HW * HR;
@@ -58,8 +66,7 @@ struct PL {
   static constexpr int CB = E + r128(3 * EP * 4);
   static constexpr int STAGE = CB + r128(EP * 4);
   static constexpr int BARS = S * STAGE;
-  static constexpr int SE = r128(BARS + 8 * S);
-  static int smem() { return SE + 3 * EP * 4; }
+  static int smem() { return BARS + 8 * S; }
 };
 
 // Stage layout of the adjoint kernel: cb and lam_E boxes (TW+8) x (TY+2) at
@@ -68,8 +75,9 @@ struct PL {
 // at (x0-4, y0-1); y: (TW+4) x (TY+2) at (x0-4, y0-1); z: (TW+4) x (TY+1) at
 // (x0-4, y0-1)) and of the H half-step at plane p-1 (x: (TW+4) x TY at
 // (x0-4, y0); y: TW x (TY+1) at (x0, y0-1); z: TW x TY at (x0, y0)).  The
-// stages' mbarriers follow the S stages; then lam_H' of plane p-1 on the
-// tile and its -x / -y halo, [3][TY+1][TW+4] at (x0-4, y0-1).
+// stages' mbarriers follow the S stages.  lam_H' of plane p-1 on the tile and
+// its -x / -y halo replaces lam_H(p) in the stage's lam_H box, once its pair's
+// thread has read that.
 // MODE 0: no CPML term in the unit; 1: z CPML terms only (tiles inside the
 // x / y interior, chunks touching a z slab); 2: every axis (the x / y ring).
 template <int TY, int S, int TW, int MODE>
@@ -90,23 +98,19 @@ struct AL {
   static constexpr int PHZ = PHY + (PXY ? r128(2 * HYP * 4) : 0);
   static constexpr int STAGE = PHZ + (PZ ? r128(2 * HZP * 4) : 0);
   static constexpr int BARS = S * STAGE;
-  static constexpr int SL = r128(BARS + 8 * S);
   // ring units: the x / y CPML profiles of the tile's cells and halo
-  static constexpr int SP = SL + r128(3 * HP * 4), SPXN = TW + 8, SPYN = TY + 4;
-  static int smem() { return PXY ? SP + 6 * (SPXN + SPYN) * 4 : SL + 3 * HP * 4; }
+  static constexpr int SP = r128(BARS + 8 * S), SPXN = TW + 8, SPYN = TY + 4;
+  static int smem() { return PXY ? SP + 6 * (SPXN + SPYN) * 4 : BARS + 8 * S; }
 };
 
-// ring_init puts the barriers at S * STAGE: the exchange arrays come after them
-static_assert(PL<8, 3, 32>::BARS == 3 * PL<8, 3, 32>::STAGE &&
-              PL<8, 3, 32>::SE >= PL<8, 3, 32>::BARS + 8 * 3, "SE after the barriers");
-static_assert(AL<8, 3, 32, 0>::SL >= AL<8, 3, 32, 0>::BARS + 8 * 3, "SL after the barriers");
-static_assert(AL<8, 3, 32, 1>::SL >= AL<8, 3, 32, 1>::BARS + 8 * 3, "SL after the barriers");
-static_assert(AL<8, 2, 32, 2>::SL >= AL<8, 2, 32, 2>::BARS + 8 * 2, "SL after the barriers");
 
 // Resident CTAs per SM the register allocation must allow (what the shared
-// memory of the default shapes allows).
+// memory of the shapes below allows).  Two stages and six (five) CTAs of the
+// adjoint's CPML-free (z-only) units against three stages and five (four):
+// 1974 against 1986 us per reverse step on 600 x 600 x 300, 218 against 230 on
+// 301 x 203 x 151.  The primal kernel is faster with three (1974 against 1983).
 template <int S, int MODE>
-constexpr int adj_ctas() { return MODE == 2 ? 4 : (MODE == 1 ? 4 : 5); }
+constexpr int adj_ctas() { return MODE == 2 ? 4 : (MODE == 1 ? 5 : 6); }
 
 // Tile and chunk of a unit.  Primal and CPML-free adjoint launches: a 3D
 // grid offset by (t0x, t0y, zc0).  z-only units (MODE 1): a 3D grid over the
@@ -119,11 +123,13 @@ constexpr int adj_ctas() { return MODE == 2 ? 4 : (MODE == 1 ? 4 : 5); }
 using namespace revf;
 
 // ============================================================== primal ===
-template <int TY, int S, int TW, bool EX>
-__global__ void __launch_bounds__(TW / 2 * (TY + 2), 6)
-k_rev_primal(const __grid_constant__ RevMaps m, StepArgs a) {
+// FULL: every cell the CTA evaluates and every neighbour lies in the interior
+// (the CPML-free units), so nothing is predicated on the cell; else the units
+// that touch the interior's edge.
+template <int TY, int S, int TW, bool EX, bool FULL>
+__device__ __forceinline__ void rev_primal_unit(const RevMaps& m, const StepArgs& a,
+                                                unsigned char* dsm) {
   typedef PL<TY, S, TW> Y;
-  extern __shared__ __align__(128) unsigned char dsm[];
   const Geo& g = a.g;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * (TW / 2) + tx;
   const int x0 = (blockIdx.x + a.t0x) * TW, y0 = (blockIdx.y + a.t0y) * TY;
@@ -136,12 +142,10 @@ k_rev_primal(const __grid_constant__ RevMaps m, StepArgs a) {
   const bool task = mainT || rowT || colT;
   const int x = colT ? x0 + TW : x0 + 2 * tx;
   const int y = mainT ? y0 + ty : (rowT ? y0 + TY : y0 + tx);
-  const bool rowok = y < g.ny;
-  const bool in0 = task && rowok && x < g.nx && x >= g.P && x < g.nx - g.P && y >= g.P &&
-                   y < g.ny - g.P;
-  const bool in1 = task && !colT && rowok && x + 1 < g.nx && x + 1 >= g.P &&
-                   x + 1 < g.nx - g.P && y >= g.P && y < g.ny - g.P;
-  auto primal_plane = [&](int p) { return p >= g.P && p < g.nz - g.P; };
+  const bool rowin = y >= g.P && y < g.ny - g.P;
+  const bool in0 = FULL ? task : task && rowin && x >= g.P && x < g.nx - g.P;
+  const bool in1 = FULL ? task : task && !colT && rowin && x + 1 >= g.P && x + 1 < g.nx - g.P;
+  auto primal_plane = [&](int p) { return FULL || (p >= g.P && p < g.nz - g.P); };
   const int p0_ = k0 - 1, p1_ = k1;
   uint64_t* bars = ring_init<S>(dsm, Y::STAGE);   // at Y::BARS
   // plane p >= k0 provides E^n(p): computed where p is interior, else the
@@ -163,13 +167,19 @@ k_rev_primal(const __grid_constant__ RevMaps m, StepArgs a) {
   if (tid == 0)
     for (int i = 0; i < S && p0_ + i <= p1_; ++i) issue(p0_ + i, dsm + i * Y::STAGE, bars + i);
   const int hb = (y - y0 + 1) * Y::HW + (x - x0 + 4);   // the pair in the Ht box
-  const int eb = (y - y0) * Y::EW + (x - x0);           // the pair in the E / cb boxes and SE
-  float* SE = reinterpret_cast<float*>(dsm + Y::SE);
+  const int eb = (y - y0) * Y::EW + (x - x0);           // the pair in the E / cb boxes
   const long long nc = g.nc;
-  float* const Fn = a.Fn;
-  const bool dy_ = y >= a.dlo[1] && y < a.dhi[1];
+  const unsigned oxy = 4u * (unsigned)(y * g.px + x);   // the pair within a plane (bytes)
+  // does the source plane meet the unit or its halo, the design box its tile?
+  const Src& sr = a.src;
+  const bool src =
+      sr.kind && (sr.axis == 0 ? sr.index >= x0 && sr.index <= x0 + TW
+                               : (sr.axis == 1 ? sr.index >= y0 && sr.index <= y0 + TY
+                                               : sr.index >= k0 && sr.index <= k1));
   const int dX = a.dhi[0] - a.dlo[0], dY = a.dhi[1] - a.dlo[1];
-  long long q = (long long)k0 * g.plane + (long long)y * g.px + x;   // plane k0 of the pair
+  const bool drow = mainT && y >= a.dlo[1] && y < a.dhi[1];
+  const bool dg0 = drow && in0 && x >= a.dlo[0] && x < a.dhi[0];
+  const bool dg1 = drow && in1 && x + 1 >= a.dlo[0] && x + 1 < a.dhi[0];
   float c_hx[2] = {0.f, 0.f}, c_hy[2] = {0.f, 0.f};   // Ht^{n+1/2}(p-1) x, y at the pair
   // primal Ht^{n-1/2}(p-1) pending: the x / y differences of E^n(p-1), E^n(p-1) x, y
   // and Ht^{n+1/2}(p-1)
@@ -180,28 +190,38 @@ k_rev_primal(const __grid_constant__ RevMaps m, StepArgs a) {
   int stg = 0;
   uint32_t par = 0;
   bool ok = true;
+  // One barrier per plane.  E^n replaces E^{n+1} in the stage's own E box (a
+  // pair's E^{n+1} is read by its own thread only); the stage of plane p - 1 is
+  // refilled after the barrier of plane p, which follows its last read.
   for (int p = p0_; p <= p1_; ++p) {
     unsigned char* st = dsm + stg * Y::STAGE;
-    if (!mbar_wait(bars + stg, par, kWaitCycles)) ok = false;
-    if (!__syncthreads_and(ok)) { ring_abort<S>(bars, stg, par, p, p1_, a.err); return; }
-    const float* Hb = reinterpret_cast<const float*>(st + Y::H);
-    const float* Eb = reinterpret_cast<const float*>(st + Y::E);
-    const float* CBb = reinterpret_cast<const float*>(st + Y::CB);
     const bool head = p < k0, tail = p == k1;
+    // lam_E^{n+1} of a design pair, on its way while the plane arrives
+    float2 l0 = {0.f, 0.f}, l1 = {0.f, 0.f}, l2 = {0.f, 0.f};
+    const bool dpl = !head && !tail && p >= a.dlo[2] && p < a.dhi[2];
+    if (dpl && (dg0 || dg1)) {
+      const float* Lp = a.L + p * g.plane + (y * g.px + x);
+      l0 = ld2(Lp, 0);
+      l1 = ld2(Lp + nc, 0);
+      l2 = ld2(Lp + 2 * nc, 0);
+    }
+    if (!mbar_wait(bars + stg, par, kWaitCycles)) ok = false;
+    const float* Hb = reinterpret_cast<const float*>(st + Y::H) + hb;
+    float* Eb = reinterpret_cast<float*>(st + Y::E) + eb;
     // ---- first half-step: E^n(p) on the task's cells ----
     float en0[2] = {0.f, 0.f}, en1[2] = {0.f, 0.f}, en2[2] = {0.f, 0.f};
     const bool need_e = !head && (primal_plane(p) || primal_plane(p - 1)) && (mainT || !tail);
     if (task && need_e) {
-      const float2 e0 = ld2(Eb, eb), e1 = ld2(Eb + Y::EP, eb), e2 = ld2(Eb + 2 * Y::EP, eb);
+      const float2 e0 = ld2(Eb, 0), e1 = ld2(Eb, Y::EP), e2 = ld2(Eb, 2 * Y::EP);
       en0[0] = e0.x; en0[1] = e0.y;
       en1[0] = e1.x; en1[1] = e1.y;
       en2[0] = e2.x; en2[1] = e2.y;
       const bool pp = primal_plane(p);
       const bool i0 = in0 && pp, i1 = in1 && pp;
-      if (i0 || i1) {
-        const float2 hx = ld2(Hb, hb), hy = ld2(Hb + Y::HP, hb), hz = ld2(Hb + 2 * Y::HP, hb);
-        const float2 hzy = ld2(Hb + 2 * Y::HP, hb - Y::HW), hxy = ld2(Hb, hb - Y::HW);
-        const float hzx = Hb[2 * Y::HP + hb - 1], hyx = Hb[Y::HP + hb - 1];
+      if (FULL || i0 || i1) {
+        const float2 hx = ld2(Hb, 0), hy = ld2(Hb, Y::HP), hz = ld2(Hb, 2 * Y::HP);
+        const float2 hzy = ld2(Hb, 2 * Y::HP - Y::HW), hxy = ld2(Hb, -Y::HW);
+        const float hzx = Hb[2 * Y::HP - 1], hyx = Hb[Y::HP - 1];
         const float d6[2] = {hz.x - hzy.x, hz.y - hzy.y}, d7[2] = {hy.x - c_hy[0], hy.y - c_hy[1]};
         const float d8[2] = {hx.x - c_hx[0], hx.y - c_hx[1]}, d9[2] = {hz.x - hzx, hz.y - hz.x};
         const float d10[2] = {hy.x - hyx, hy.y - hy.x}, d11[2] = {hx.x - hxy.x, hx.y - hxy.y};
@@ -212,7 +232,7 @@ k_rev_primal(const __grid_constant__ RevMaps m, StepArgs a) {
           c1[c] = d8[c] - d9[c];
           c2[c] = d10[c] - d11[c];
         }
-        if (a.src.kind) {
+        if (src) {
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
             const float w = (c == 0 ? i0 : i1) ? src_wt(a.src, x + c, y, p) : 0.f;
@@ -224,103 +244,120 @@ k_rev_primal(const __grid_constant__ RevMaps m, StepArgs a) {
             }
           }
         }
-        const float2 cb2 = ld2(CBb, eb);
+        const float2 cb2 = ld2(reinterpret_cast<const float*>(st + Y::CB), eb);
         const float cbv[2] = {cb2.x, cb2.y};
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          if (c == 0 ? i0 : i1) {
+          if (FULL || (c == 0 ? i0 : i1)) {
             en0[c] = __fsub_rn(en0[c], inc_of<EX>(__fmul_rn(cbv[c], c0[c]), a));
             en1[c] = __fsub_rn(en1[c], inc_of<EX>(__fmul_rn(cbv[c], c1[c]), a));
             en2[c] = __fsub_rn(en2[c], inc_of<EX>(__fmul_rn(cbv[c], c2[c]), a));
           }
         }
-        if (mainT && !tail) {
-          ST2(Fn, q, en0[0], en0[1], i0, i1);
-          ST2(Fn + nc, q, en1[0], en1[1], i0, i1);
-          ST2(Fn + 2 * nc, q, en2[0], en2[1], i0, i1);
+        if (!tail) {
+          *reinterpret_cast<float2*>(Eb) = make_float2(en0[0], en0[1]);
+          *reinterpret_cast<float2*>(Eb + Y::EP) = make_float2(en1[0], en1[1]);
+          *reinterpret_cast<float2*>(Eb + 2 * Y::EP) = make_float2(en2[0], en2[1]);
+          if (mainT) {
+            float* O = a.Fn + p * g.plane;
+            put2(a, O, oxy, en0[0], en0[1], FULL || i0, FULL || i1);
+            put2(a, O + nc, oxy, en1[0], en1[1], FULL || i0, FULL || i1);
+            put2(a, O + 2 * nc, oxy, en2[0], en2[1], FULL || i0, FULL || i1);
+          }
           // dL/dcb on the design box: lam_E^{n+1} . (curl Ht - J)
-          if (dy_ && p >= a.dlo[2] && p < a.dhi[2]) {
+          if (dpl && (dg0 || dg1)) {
+            const float lx[2] = {l0.x, l0.y}, ly[2] = {l1.x, l1.y}, lz[2] = {l2.x, l2.y};
+            double* gp = a.gacc + ((long long)(p - a.dlo[2]) * dY + (y - a.dlo[1])) * dX +
+                         (x - a.dlo[0]);
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-              const int xc = x + c;
-              if ((c == 0 ? i0 : i1) && xc >= a.dlo[0] && xc < a.dhi[0]) {
-                const long long qc = q + c;
-                const float s =
-                        grad_term(a.L[qc], a.L[nc + qc], a.L[2 * nc + qc], c0[c], c1[c], c2[c]);
-                const long long qd =
-                    ((long long)(p - a.dlo[2]) * dY + (y - a.dlo[1])) * dX + (xc - a.dlo[0]);
+              if (c == 0 ? dg0 && i0 : dg1 && i1) {
+                const float s = grad_term(lx[c], ly[c], lz[c], c0[c], c1[c], c2[c]);
 #ifdef FDTD_BOUNDS_CHECK
+                const long long qd = gp + c - a.gacc;
                 if (qd < 0 || qd >= (long long)dX * dY * (a.dhi[2] - a.dlo[2])) {
                   atomicOr(a.err, ERR_BOUNDS);
                   continue;
                 }
 #endif
-                atomicAdd(a.gacc + qd, (double)s);
+                atomicAdd(gp + c, (double)s);
               }
             }
           }
         }
       }
-      if (!tail && primal_plane(p)) {
-        *reinterpret_cast<float2*>(SE + eb) = make_float2(en0[0], en0[1]);
-        *reinterpret_cast<float2*>(SE + Y::EP + eb) = make_float2(en1[0], en1[1]);
-        *reinterpret_cast<float2*>(SE + 2 * Y::EP + eb) = make_float2(en2[0], en2[1]);
-      }
     }
     // Ht^{n+1/2}(p) x, y at the task's cells for the next plane's z differences
     if (task && !tail && (head ? primal_plane(p + 1) : (primal_plane(p) || primal_plane(p + 1)))) {
-      const float2 hx = ld2(Hb, hb), hy = ld2(Hb + Y::HP, hb);
+      const float2 hx = ld2(Hb, 0), hy = ld2(Hb, Y::HP);
       c_hx[0] = hx.x; c_hx[1] = hx.y;
       c_hy[0] = hy.x; c_hy[1] = hy.y;
     }
-    __syncthreads();   // E^n(p) of the tile and its halo is in SE
+    // E^n(p) of the tile and its halo is in the stage; a wait that gave up ends
+    // the CTA here
+    if (!__syncthreads_and(ok)) { ring_abort<S>(bars, stg, par, p, p1_, a.err); return; }
+    if (tid == 0 && p > p0_ && p - 1 + S <= p1_) {   // the stage of plane p - 1 is free
+      const int sp = stg == 0 ? S - 1 : stg - 1;
+      issue(p - 1 + S, dsm + sp * Y::STAGE, bars + sp);
+    }
     // ---- second half-step, one plane behind: Ht^{n-1/2}(p-1) ----
     if (mainT && !head) {
-      if (p > k0 && (c_pr0 || c_pr1)) {
+      if (p > k0 && (FULL || c_pr0 || c_pr1)) {
         const float d1[2] = {en1[0] - c_ey[0], en1[1] - c_ey[1]};
         const float d2[2] = {en0[0] - c_ex[0], en0[1] - c_ex[1]};
-        const long long qm = q - g.plane;
         auto inc = [&](float cc) { return inc_of<EX>(__fmul_rn(g.S, cc), a); };
-        ST2(Fn + 3 * nc, qm, __fadd_rn(c_h0[0], inc(c_d0[0] - d1[0])),
-            __fadd_rn(c_h0[1], inc(c_d0[1] - d1[1])), c_pr0, c_pr1);
-        ST2(Fn + 4 * nc, qm, __fadd_rn(c_h1[0], inc(d2[0] - c_d3[0])),
-            __fadd_rn(c_h1[1], inc(d2[1] - c_d3[1])), c_pr0, c_pr1);
-        ST2(Fn + 5 * nc, qm, __fadd_rn(c_h2[0], inc(c_d4[0] - c_d5[0])),
-            __fadd_rn(c_h2[1], inc(c_d4[1] - c_d5[1])), c_pr0, c_pr1);
+        float* O = a.Fn + 3 * nc + (p - 1) * g.plane;
+        put2(a, O, oxy, __fadd_rn(c_h0[0], inc(c_d0[0] - d1[0])),
+             __fadd_rn(c_h0[1], inc(c_d0[1] - d1[1])), FULL || c_pr0, FULL || c_pr1);
+        put2(a, O + nc, oxy, __fadd_rn(c_h1[0], inc(d2[0] - c_d3[0])),
+             __fadd_rn(c_h1[1], inc(d2[1] - c_d3[1])), FULL || c_pr0, FULL || c_pr1);
+        put2(a, O + 2 * nc, oxy, __fadd_rn(c_h2[0], inc(c_d4[0] - c_d5[0])),
+             __fadd_rn(c_h2[1], inc(c_d4[1] - c_d5[1])), FULL || c_pr0, FULL || c_pr1);
       }
       if (!tail) {
         const bool pp = primal_plane(p);
         c_pr0 = pp && in0;
         c_pr1 = pp && in1;
-        if (c_pr0 || c_pr1) {   // x and y differences of E^n(p) now, z differences next plane
-          const float2 ezy = ld2(SE + 2 * Y::EP, eb + Y::EW), exy = ld2(SE, eb + Y::EW);
-          const float ezx = SE[2 * Y::EP + eb + 2], eyx = SE[Y::EP + eb + 2];
+        if (FULL || c_pr0 || c_pr1) {   // x and y differences of E^n(p) now, z next plane
+          const float2 ezy = ld2(Eb, 2 * Y::EP + Y::EW), exy = ld2(Eb, Y::EW);
+          const float ezx = Eb[2 * Y::EP + 2], eyx = Eb[Y::EP + 2];
           c_d0[0] = ezy.x - en2[0]; c_d0[1] = ezy.y - en2[1];
           c_d3[0] = en2[1] - en2[0]; c_d3[1] = ezx - en2[1];
           c_d4[0] = en1[1] - en1[0]; c_d4[1] = eyx - en1[1];
           c_d5[0] = exy.x - en0[0]; c_d5[1] = exy.y - en0[1];
           c_ex[0] = en0[0]; c_ex[1] = en0[1];
           c_ey[0] = en1[0]; c_ey[1] = en1[1];
-          const float2 h0 = ld2(Hb, hb), h1 = ld2(Hb + Y::HP, hb), h2 = ld2(Hb + 2 * Y::HP, hb);
+          const float2 h0 = ld2(Hb, 0), h1 = ld2(Hb, Y::HP), h2 = ld2(Hb, 2 * Y::HP);
           c_h0[0] = h0.x; c_h0[1] = h0.y;
           c_h1[0] = h1.x; c_h1[1] = h1.y;
           c_h2[0] = h2.x; c_h2[1] = h2.y;
         }
-        q += g.plane;
       }
     }
-    __syncthreads();   // SE and the stage are free again
-    if (tid == 0 && p + S <= p1_) issue(p + S, st, bars + stg);
     if (++stg == S) { stg = 0; par ^= 1u; }
   }
+}
+
+template <int TY, int S, int TW, bool EX>
+__global__ void __launch_bounds__(TW / 2 * (TY + 2), 6)
+k_rev_primal(const __grid_constant__ RevMaps m, const __grid_constant__ StepArgs a) {
+  extern __shared__ __align__(128) unsigned char dsm[];
+  const int tix = blockIdx.x + a.t0x, tiy = blockIdx.y + a.t0y, cz = blockIdx.z + a.zc0;
+  const RevUnits& U = a.U;
+  if (tix >= U.ix0 && tix < U.ix1 && tiy >= U.iy0 && tiy < U.iy1 && cz >= U.iz0 && cz < U.iz1)
+    rev_primal_unit<TY, S, TW, EX, true>(m, a, dsm);
+  else
+    rev_primal_unit<TY, S, TW, EX, false>(m, a, dsm);
 }
 
 // ============================================================= adjoint ===
 template <int TY, int S, int TW, int MODE>
 __global__ void __launch_bounds__(TW / 2 * (TY + 2), (adj_ctas<S, MODE>()))
-k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
+k_rev_adjoint(const __grid_constant__ RevMaps m, const __grid_constant__ StepArgs a,
+              const __grid_constant__ RevUnits U) {
   typedef AL<TY, S, TW, MODE> Y;
   constexpr bool PXY = Y::PXY, PZ = Y::PZ;
+  constexpr bool IN = !PXY;   // the tile and its halo lie inside the x / y interior
   extern __shared__ __align__(128) unsigned char dsm[];
   const Geo& g = a.g;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * (TW / 2) + tx;
@@ -343,8 +380,8 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
   const int x = colT ? x0 - 2 : x0 + 2 * tx;
   const int y = mainT ? y0 + ty : (rowT ? y0 - 1 : y0 + tx);
   const bool rowok = y >= 0 && y < g.ny;
-  const bool ok0 = task && rowok && x >= 0 && x < g.nx;
-  const bool ok1 = task && rowok && x + 1 >= 0 && x + 1 < g.nx;
+  const bool ok0 = task && (IN || (rowok && x >= 0 && x < g.nx));
+  const bool ok1 = task && (IN || (rowok && x + 1 >= 0 && x + 1 < g.nx));
   const bool v0 = mainT && ok0, v1 = mainT && ok1;   // cells this thread stores
   const int p0_ = k0 - 1, p1_ = k1;
   // ring units: the x / y CPML profiles the tile's cells and halo read,
@@ -421,12 +458,14 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
   }
   const int wb = (y - y0 + 1) * Y::WW + (x - x0 + 4);   // the pair in the cb / lam_E boxes
   const int lb = (y - y0 + 1) * Y::HW + (x - x0 + 4);   // the pair in the lam_H box and SL
-  float* SL = reinterpret_cast<float*>(dsm + Y::SL);
   const float S_ = g.S;
   const long long nc = g.nc;
   float* const Ln = a.Ln;
   float* const lpB = a.psiB;
-  long long q = (long long)k0 * g.plane + (long long)y * g.px + x;   // plane k0 of the pair
+  const unsigned oxy = 4u * (unsigned)(y * g.px + x);   // the pair within a plane (bytes)
+  // the same in the x and y auxiliary arrays (z: as in the fields)
+  const unsigned opx = PXY ? 4u * (unsigned)(y * a.pl.ax[0].d0 + psi_map(a.pl.ax[0], x)) : 0u;
+  const unsigned opy = PXY ? 4u * (unsigned)(psi_map(a.pl.ax[1], y) * a.pl.ax[1].d0 + x) : 0u;
   // lam_H'(p-1): own lam_H x, y, the +z terms pending and the completed x / y parts;
   // lam_Hz'(p-1) complete
   float c_lhx[2] = {0.f, 0.f}, c_lhy[2] = {0.f, 0.f}, c_o8[2] = {0.f, 0.f}, c_o7[2] = {0.f, 0.f};
@@ -440,10 +479,10 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
   for (int p = p0_; p <= p1_; ++p) {
     unsigned char* st = dsm + stg * Y::STAGE;
     if (!mbar_wait(bars + stg, par, kWaitCycles)) ok = false;
-    if (!__syncthreads_and(ok)) { ring_abort<S>(bars, stg, par, p, p1_, a.err); return; }
     const float* CBb = reinterpret_cast<const float*>(st + Y::CB);
     const float* LEb = reinterpret_cast<const float*>(st + Y::LE);
     const float* LHb = reinterpret_cast<const float*>(st + Y::LH);
+    float* SL = reinterpret_cast<float*>(st + Y::LH);
     const bool head = p < k0, tail = p == k1;
     const bool zs = PZ && inz(p) && in_slab(p, g.nz, g.P);
     float fx[2] = {0.f, 0.f}, fy[2] = {0.f, 0.f};   // lam_Hx', lam_Hy' of plane p-1
@@ -466,7 +505,7 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
                         wz = __fmul_rn(cbv[c], own_le[2][c]);
             o6[c] = wx; o11[c] = -wz; o7[c] = -wx; o8[c] = wy; o9[c] = -wy; o10[c] = wz;
           }
-          if (y + 1 < g.ny) {
+          if (IN || y + 1 < g.ny) {
             const float2 cy2 = ld2(CBb, wb + Y::WW);
             const float2 ly = ld2(LEb, wb + Y::WW), lz = ld2(LEb + 2 * Y::WP, wb + Y::WW);
             n6[0] = __fmul_rn(cy2.x, ly.x);
@@ -474,7 +513,7 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
             n11[0] = __fmul_rn(-cy2.x, lz.x);
             n11[1] = __fmul_rn(-cy2.y, lz.y);
           }
-          if (x + 2 < g.nx) {
+          if (IN || x + 2 < g.nx) {
             const float c2 = CBb[wb + 2];
             n9x = __fmul_rn(-c2, LEb[Y::WP + wb + 2]);
             n10x = __fmul_rn(c2, LEb[2 * Y::WP + wb + 2]);
@@ -495,9 +534,9 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
                 o11[c] = adj(o11[c], q1[c], by, ay, ky, &s11[c]);
               }
               if (!head && (v0 || v1)) {
-                const long long qyy = psi_ix<1>(a.pl, 2, x, y, p);
-                ST2(lpB, qyy, s6[0], s6[1], v0, v1);
-                ST2(lpB + a.pl.ax[1].cs, qyy, s11[0], s11[1], v0, v1);
+                float* O = lpB + a.pl.ax[1].off + 2 * a.pl.ax[1].cs + p * a.pl.ax[1].ps;
+                put2(a, O, opy, s6[0], s6[1], v0, v1);
+                put2(a, O + a.pl.ax[1].cs, opy, s11[0], s11[1], v0, v1);
               }
             }
             if (sy1) {
@@ -530,9 +569,9 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
               o10[1] = adj(o10[1], p1.y, b, aa, kk, &s10[1]);
             }
             if (!head && ((v0 && sx0) || (v1 && sx1))) {
-              const long long qxx = psi_ix<0>(a.pl, 2, x, y, p);
-              ST2(lpB, qxx, s9[0], s9[1], v0 && sx0, v1 && sx1);
-              ST2(lpB + a.pl.ax[0].cs, qxx, s10[0], s10[1], v0 && sx0, v1 && sx1);
+              float* O = lpB + a.pl.ax[0].off + 2 * a.pl.ax[0].cs + p * a.pl.ax[0].ps;
+              put2(a, O, opx, s9[0], s9[1], v0 && sx0, v1 && sx1);
+              put2(a, O + a.pl.ax[0].cs, opx, s10[0], s10[1], v0 && sx0, v1 && sx1);
             }
             if (sx2) {
               const float b = spx(PR_BE, x + 2), aa = spx(PR_AE, x + 2),
@@ -555,9 +594,9 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
             o8[c] = adj(o8[c], q1[c], b, aa, kv, &s8[c]);
           }
           if (!head && (v0 || v1)) {
-            const long long qz = psi_ix<2>(a.pl, 2, x, y, p);
-            ST2(lpB, qz, s7[0], s7[1], v0, v1);
-            ST2(lpB + a.pl.ax[2].cs, qz, s8[0], s8[1], v0, v1);
+            float* O = lpB + a.pl.ax[2].off + 2 * a.pl.ax[2].cs + psi_map(a.pl.ax[2], p) * a.pl.ax[2].ps;
+            put2(a, O, oxy, s7[0], s7[1], v0, v1);
+            put2(a, O + a.pl.ax[2].cs, oxy, s8[0], s8[1], v0, v1);
           }
         }
         // cell 0's +x terms are cell 1's own terms
@@ -577,10 +616,10 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
           *reinterpret_cast<float2*>(SL + Y::HP + lb) = make_float2(fy[0], fy[1]);
           *reinterpret_cast<float2*>(SL + 2 * Y::HP + lb) = make_float2(c_lhz[0], c_lhz[1]);
           if (p - 1 >= k0) {
-            const long long qm = q - g.plane;
-            ST2(Ln + 3 * nc, qm, fx[0], fx[1], v0, v1);
-            ST2(Ln + 4 * nc, qm, fy[0], fy[1], v0, v1);
-            ST2(Ln + 5 * nc, qm, c_lhz[0], c_lhz[1], v0, v1);
+            float* O = Ln + 3 * nc + (p - 1) * g.plane;
+            put2(a, O, oxy, fx[0], fx[1], v0, v1);
+            put2(a, O + nc, oxy, fy[0], fy[1], v0, v1);
+            put2(a, O + 2 * nc, oxy, c_lhz[0], c_lhz[1], v0, v1);
           }
         }
         c_lhx[0] = lh0.x; c_lhx[1] = lh0.y;
@@ -622,13 +661,15 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
         *reinterpret_cast<float2*>(SL + lb) = make_float2(fx[0], fx[1]);
         *reinterpret_cast<float2*>(SL + Y::HP + lb) = make_float2(fy[0], fy[1]);
         *reinterpret_cast<float2*>(SL + 2 * Y::HP + lb) = make_float2(c_lhz[0], c_lhz[1]);
-        const long long qm = q - g.plane;
-        ST2(Ln + 3 * nc, qm, fx[0], fx[1], v0, v1);
-        ST2(Ln + 4 * nc, qm, fy[0], fy[1], v0, v1);
-        ST2(Ln + 5 * nc, qm, c_lhz[0], c_lhz[1], v0, v1);
+        float* O = Ln + 3 * nc + (p - 1) * g.plane;
+        put2(a, O, oxy, fx[0], fx[1], v0, v1);
+        put2(a, O + nc, oxy, fy[0], fy[1], v0, v1);
+        put2(a, O + 2 * nc, oxy, c_lhz[0], c_lhz[1], v0, v1);
       }
     }
-    __syncthreads();   // lam_H'(p-1) of the tile and its halo is in SL
+    // lam_H'(p-1) of the tile and its halo is in SL; a wait that gave up ends the
+    // CTA here
+    if (!__syncthreads_and(ok)) { ring_abort<S>(bars, stg, par, p, p1_, a.err); return; }
     // ---- transpose of the H half-step, one plane behind: lam_E'(p-1) ----
     if (mainT && !head) {
       if (p - 1 >= k0) {
@@ -653,8 +694,8 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
           m5[0] = __fmul_rn(S_, lzy.x);  m5[1] = __fmul_rn(S_, lzy.y);
         }
         float m3x = __fmul_rn(S_, SL[Y::HP + lb - 1]), m4x = __fmul_rn(-S_, SL[2 * Y::HP + lb - 1]);   // -x of cell 0
-        if (y == 0) { m0[0] = 0.f; m0[1] = 0.f; m5[0] = 0.f; m5[1] = 0.f; }
-        if (x == 0) { m3x = 0.f; m4x = 0.f; }
+        if (!IN && y == 0) { m0[0] = 0.f; m0[1] = 0.f; m5[0] = 0.f; m5[1] = 0.f; }
+        if (!IN && x == 0) { m3x = 0.f; m4x = 0.f; }
         const int pm = p - 1;
         {
           if (PXY && (hy || hym)) {
@@ -670,9 +711,9 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
                 o0[c] = adj(o0[c], q0[c], by, ay, ky, &s4[c]);
                 o5[c] = adj(o5[c], q1[c], by, ay, ky, &s5[c]);
               }
-              const long long qyy = psi_ix<1>(a.pl, 0, x, y, pm);
-              ST2(lpB, qyy, s4[0], s4[1], v0, v1);
-              ST2(lpB + a.pl.ax[1].cs, qyy, s5[0], s5[1], v0, v1);
+              float* O = lpB + a.pl.ax[1].off + 0 * a.pl.ax[1].cs + pm * a.pl.ax[1].ps;
+              put2(a, O, opy, s4[0], s4[1], v0, v1);
+              put2(a, O + a.pl.ax[1].cs, opy, s5[0], s5[1], v0, v1);
             }
             if (hym) {
               const float bym = spy(PR_BH, y - 1), aym = spy(PR_AH, y - 1),
@@ -703,9 +744,9 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
               o3[1] = adj(o3[1], p0.y, b, aa, kk, &s0[1]);
               o4[1] = adj(o4[1], p1.y, b, aa, kk, &s1[1]);
             }
-            const long long qxx = psi_ix<0>(a.pl, 0, x, y, pm);
-            ST2(lpB, qxx, s0[0], s0[1], hx0, hx1);
-            ST2(lpB + a.pl.ax[0].cs, qxx, s1[0], s1[1], hx0, hx1);
+            float* O = lpB + a.pl.ax[0].off + 0 * a.pl.ax[0].cs + pm * a.pl.ax[0].ps;
+            put2(a, O, opx, s0[0], s0[1], hx0, hx1);
+            put2(a, O + a.pl.ax[0].cs, opx, s1[0], s1[1], hx0, hx1);
             if (hxm) {
               const float b = spx(PR_BH, x - 1), aa = spx(PR_AH, x - 1),
                           kk = spx(PR_KH, x - 1);
@@ -726,19 +767,19 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
               o1[c] = adj(o1[c], q0[c], b, aa, kv, &s8[c]);
               o2[c] = adj(o2[c], q1[c], b, aa, kv, &s9[c]);
             }
-            const long long qz = psi_ix<2>(a.pl, 0, x, y, pm);
-            ST2(lpB, qz, s8[0], s8[1], v0, v1);
-            ST2(lpB + a.pl.ax[2].cs, qz, s9[0], s9[1], v0, v1);
+            float* O = lpB + a.pl.ax[2].off + 0 * a.pl.ax[2].cs + psi_map(a.pl.ax[2], pm) * a.pl.ax[2].ps;
+            put2(a, O, oxy, s8[0], s8[1], v0, v1);
+            put2(a, O + a.pl.ax[2].cs, oxy, s9[0], s9[1], v0, v1);
           }
         }
         // cell 1's -x terms are cell 0's own terms
         const float m3[2] = {m3x, o3[0]}, m4[2] = {m4x, o4[0]};
-        const long long qm = q - g.plane;
-        ST2(Ln, qm, c_le0[0] + ((c_m2[0] - o2[0]) + (m5[0] - o5[0])),
+        float* O = Ln + (p - 1) * g.plane;
+        put2(a, O, oxy, c_le0[0] + ((c_m2[0] - o2[0]) + (m5[0] - o5[0])),
             c_le0[1] + ((c_m2[1] - o2[1]) + (m5[1] - o5[1])), v0, v1);
-        ST2(Ln + nc, qm, c_le1[0] + ((c_m1[0] - o1[0]) + (m4[0] - o4[0])),
+        put2(a, O + nc, oxy, c_le1[0] + ((c_m1[0] - o1[0]) + (m4[0] - o4[0])),
             c_le1[1] + ((c_m1[1] - o1[1]) + (m4[1] - o4[1])), v0, v1);
-        ST2(Ln + 2 * nc, qm, c_le2[0] + ((m0[0] - o0[0]) + (m3[0] - o3[0])),
+        put2(a, O + 2 * nc, oxy, c_le2[0] + ((m0[0] - o0[0]) + (m3[0] - o3[0])),
             c_le2[1] + ((m0[1] - o0[1]) + (m3[1] - o3[1])), v0, v1);
         // the -z terms plane p needs are this plane's own z-terms
 #pragma unroll
@@ -783,7 +824,6 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, StepArgs a, RevUnits U) {
         c_le1[c] = own_le[1][c];
         c_le2[c] = own_le[2][c];
       }
-      if (!head) q += g.plane;
     }
     __syncthreads();   // SL and the stage are free again
     if (tid == 0 && p + S <= p1_) issue(p + S, st, bars + stg);
@@ -812,9 +852,9 @@ static cudaError_t launch_rev_fused_t(int which, const RevMaps& m, const StepArg
         return launch_rf(k_rev_primal<TY, 3, TW, true>, grid, block, PL<TY, 3, TW>::smem(), s, m, a);
       return launch_rf(k_rev_primal<TY, 3, TW, false>, grid, block, PL<TY, 3, TW>::smem(), s, m, a);
     case 1:
-      return launch_rf(k_rev_adjoint<TY, 3, TW, 0>, grid, block, AL<TY, 3, TW, 0>::smem(), s, m, a, U);
+      return launch_rf(k_rev_adjoint<TY, 2, TW, 0>, grid, block, AL<TY, 2, TW, 0>::smem(), s, m, a, U);
     case 2:
-      return launch_rf(k_rev_adjoint<TY, 3, TW, 1>, grid, block, AL<TY, 3, TW, 1>::smem(), s, m, a, U);
+      return launch_rf(k_rev_adjoint<TY, 2, TW, 1>, grid, block, AL<TY, 2, TW, 1>::smem(), s, m, a, U);
     case 3:
       return launch_rf(k_rev_adjoint<TY, 2, TW, 2>, grid, block, AL<TY, 2, TW, 2>::smem(), s, m, a, U);
   }
@@ -827,6 +867,7 @@ cudaError_t launch_rev_fused(int which, const RevMaps& m, const StepArgs& a, con
   if (a.tile_y != TY || a.tile_x != TW) return cudaErrorInvalidValue;
   dim3 grid(0, 0, 0);
   StepArgs b = a;
+  b.U = U;
   const int nzin = U.iz1 - U.iz0;
   switch (which) {
     case 0:

@@ -133,6 +133,25 @@ __device__ __forceinline__ bool store_ok(const StepArgs& a, const float* p) {
 #define ST2(p, q, u, v, f0, f1) st2(p, q, u, v, f0, f1)
 #endif
 
+// Store the pair (u, v) at a byte offset within a plane of a component, whose
+// base is the same for the whole CTA: the base stays in uniform registers and
+// the address costs one addition.  (A plane of a grid that fits the device is
+// far below 4 GB.)
+__device__ __forceinline__ void put2(const StepArgs& a, float* plane, unsigned off, float u, float v,
+                                     bool f0, bool f1) {
+  float* p = reinterpret_cast<float*>(reinterpret_cast<char*>(plane) + off);
+#ifdef FDTD_BOUNDS_CHECK
+  f0 = f0 && store_ok(a, p);
+  f1 = f1 && store_ok(a, p + 1);
+#endif
+  if (f0 && f1) {
+    *reinterpret_cast<float2*>(p) = make_float2(u, v);
+  } else {
+    if (f0) p[0] = u;
+    if (f1) p[1] = v;
+  }
+}
+
 // Forward CPML recursion of one derivative d (Eq. 5 form): the updated psi
 // goes to *s, the stretched derivative is returned.
 __device__ __forceinline__ float cpml(float d, float psi_old, float b, float a, float kv, float* s) {
