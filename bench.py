@@ -385,9 +385,6 @@ def sampled_breakdown(A, fdtd, args, w, rec, dev, flush):
     torch.cuda.synchronize()
     per_step = {"record": 1.0 / rec.k, "fwd_2step": 0.5}
     kb = kernel_bytes(w)
-    other = "fwd_fused" in ktimes or "fwd_2step" in ktimes
-    if other:   # the split half-steps ran only the other units
-        kb = {k: v for k, v in kb.items() if k not in ("fwd_h", "fwd_e")}
     step_ms = statistics.median(loop_ms) / ws_.n_steps
     kern = {}
     for name, lst in ktimes.items():
@@ -398,10 +395,8 @@ def sampled_breakdown(A, fdtd, args, w, rec, dev, flush):
         if name in kb:
             d["own_bytes"] = kb[name]
             d["own_gbs"] = kb[name] / (avg / 1e3) / 1e9
-        if name in ("fwd_h", "fwd_e") and "fwd_fused" in ktimes:
-            d["units"] = "the CPML units of the fused forward step"
-        if name in ("fwd_h", "fwd_e") and "fwd_2step" in ktimes:
-            d["units"] = "the units outside the deep box, one time step per launch"
+        if name == "fwd_fused" and "fwd_2step" in ktimes:
+            d["units"] = "the units outside the deep box, one time step (four launches)"
         if name == "fwd_2step":
             d["units"] = "the deep units, two time steps per launch"
         kern[name] = d

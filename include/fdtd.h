@@ -309,9 +309,11 @@ enum {
                                    off.  Injects no fault: the wait is the same bounded wait
                                    as fdtd_selftest_wait */
   FDTD_OPT_REVERSE = 15,        /* kernel 5: how a reverse time step runs.  0 (default) =
-                                   automatic: fused with 32 x 8 tiles when at most half of
-                                   the (tile, z chunk) units carry CPML terms (see
-                                   fdtd_reverse_units), else split; 1 = split:
+                                   automatic: small grids the direct half-steps (as in
+                                   FDTD_OPT_FORWARD); from 9 million cells on fused with
+                                   32 x 8 tiles when at most half of the (tile, z chunk)
+                                   units carry CPML terms (see fdtd_reverse_units), else
+                                   split; 1 = split:
                                    a reverse E phase and a reverse H phase, each updating the
                                    primal and the adjoint fields in place; 2 = fused: one
                                    launch for the primal fields (both inverse half-steps,
@@ -320,41 +322,41 @@ enum {
                                    each reading every field once and writing it once into
                                    the other buffer of a ping-pong pair (the workspace holds
                                    a second field and adjoint buffer); FDTD_EINVAL at
-                                   fdtd_forward with other tiles.  Results agree with the
-                                   split phases: primal fields bit for bit, gradients to
-                                   rounding */
+                                   fdtd_forward with other tiles.  The fields and the
+                                   gradient are bit-identical to the split phases' */
   FDTD_OPT_FORWARD = 16,        /* kernel 5: how a forward time step runs.  0 (default) =
-                                   automatic: where at most half of the (tile, z chunk)
-                                   units carry CPML terms, two steps per pass (3) where it
-                                   can run (below), else fused where it can run; split
-                                   elsewhere; 1 = split: an H and an E half-step launch, each
-                                   updating the fields in place; 2 = fused: the units
-                                   without a CPML term (fdtd_reverse_units' CPML-free box)
-                                   run both half-steps in one launch that reads every field
-                                   once and writes it once into the other buffer of a
-                                   ping-pong pair, and the other units run the split
-                                   half-steps from and into the same pair.  Needs 32 x 8
-                                   tiles, such units, and the source and the detector
-                                   outside them; else FDTD_EINVAL at fdtd_forward.  The
-                                   fields are bit-identical to the split half-steps'; 3 =
-                                   two steps per pass (temporal blocking, not part of the
-                                   paper's method): the deep units (fdtd_deep_units: no
-                                   CPML term on their cells or a two-cell halo) run time
-                                   steps n and n + 1 in one launch that reads E^n,
-                                   Ht^{n-1/2} and cb once and writes E^{n+2}, Ht^{n+3/2}
-                                   once into the other buffer of the pair, plus the
-                                   intermediate level on the one-cell frame of the deep
-                                   box into a third field buffer; the other units run the
-                                   split half-steps one step at a time through that
-                                   buffer.  Needs 32 x 8 tiles, deep units, and the source
-                                   and the detectors two cells or more away from them;
-                                   else FDTD_EINVAL at fdtd_forward.  An odd step count
-                                   runs its first step as split half-steps over every
-                                   unit.  The fields and the tape are bit-identical to
-                                   the split half-steps' */
+                                   automatic: small grids the direct half-steps (one pair of
+                                   cells per thread; only with the default shape options),
+                                   larger ones the split half-steps, from 12 million cells
+                                   on two steps per pass (3) where it can run (below), at
+                                   most half of the (tile, z chunk) units carrying CPML
+                                   terms, else the fused step; 1 = split: an H and an E
+                                   half-step launch, each updating the fields in place;
+                                   2 = fused: both half-steps of a unit in one launch that
+                                   reads every field once and writes it once into the other
+                                   buffer of a ping-pong pair (launches by the CPML axes a
+                                   unit can meet).  Asked for by name it needs 32 x 8 tiles,
+                                   units without a CPML term (fdtd_reverse_units' CPML-free
+                                   box), and the source and the detector outside them; else
+                                   FDTD_EINVAL at fdtd_forward.  The fields are
+                                   bit-identical to the split half-steps'; 3 = two steps
+                                   per pass (temporal blocking, not part of the paper's
+                                   method): the deep units (fdtd_deep_units: no CPML term
+                                   on their cells or a two-cell halo) run time steps n and
+                                   n + 1 in one launch that reads E^n, Ht^{n-1/2} and cb
+                                   once and writes E^{n+2}, Ht^{n+3/2} once into the other
+                                   buffer of the pair, plus the intermediate level on the
+                                   one-cell frame of the deep box into a third field buffer;
+                                   the other units run the fused step one time step at a
+                                   time through that buffer.  Needs 32 x 8 tiles, deep
+                                   units, and the source and the detectors two cells or
+                                   more away from them; else FDTD_EINVAL at fdtd_forward.
+                                   An odd step count runs its first step as a fused step
+                                   over every unit.  The fields and the tape are
+                                   bit-identical to the split half-steps' */
   FDTD_OPT_ZCHUNK_FWD2 = 17     /* kernel 5 with FDTD_OPT_FORWARD = 3: z planes per CTA of
                                    the two-step pass (-1 or 0, the default: sixteen chunks
-                                   of the other units' split half-steps, whose chunks are
+                                   of the other units' fused step, whose chunks are
                                    FDTD_OPT_ZCHUNK_FWD planes if > 0, else FDTD_OPT_ZCHUNK);
                                    a chunk streams two planes below and one above it */
 };

@@ -521,13 +521,45 @@ static bool direct_reverse(const fdtd_handle* h) {
          (long long)h->nx * h->ny * h->nz <= kDirectReverseCells;
 }
 
+// How a forward and a reverse run.  Named forms (FDTD_OPT_FORWARD 1-3,
+// FDTD_OPT_REVERSE 1-2) run as asked, where they may.  Automatic: the direct
+// half-steps on small grids; the split ones on grids that partly stay in the L2
+// cache, where the fused launches' second buffers cost more than the second read
+// they save; beyond, two steps per pass where they may run (two_step_forward),
+// else the fused step, and the fused reverse step where it may (fused_reverse).  us
+// per step, forward split / fused / two steps: 60 / 73 / 85 on 200 x 200 x 100 (4 M
+// cells), 127 / 132 / 141 on 301 x 203 x 151 (9.2 M), 144 / 147 / 133 on 300 x 300 x
+// 120 (10.8 M), 176 / 175 / 155 on 300 x 300 x 150 (13.5 M), 407 / - / 324 on 411 x
+// 389 x 203 (32 M); reverse split / fused: 104 / 120 (4 M), 195 / 199 (7.8 M), 224 /
+// 220 (9.2 M), 320 / 313 (13.5 M), 725 / 638 (32 M).  An option that names another
+// shape of the split half-steps leaves the choice to the units' CPML share alone.
+enum ForwardForm { kSplit, kDirect, kFusedStep, kTwoStep };
+static const long long kFusedForwardCells = 12000000, kFusedReverseCells = 9000000;
+static long long cells_of(const fdtd_handle* h) { return (long long)h->nx * h->ny * h->nz; }
+static ForwardForm forward_form(const fdtd_handle* h) {
+  if (h->opt_kernel != 5 || h->opt_forward == 1) return kSplit;
+  if (direct_forward(h)) return kDirect;
+  if (two_step_forward(h) && (h->opt_forward == 3 || !direct_shape(h) ||
+                              cells_of(h) >= kFusedForwardCells))
+    return kTwoStep;
+  if (fused_forward(h) && (h->opt_forward == 2 || !direct_shape(h))) return kFusedStep;
+  return h->opt_forward == 0 && direct_shape(h) && cells_of(h) >= kFusedForwardCells ? kFusedStep
+                                                                                     : kSplit;
+}
+static bool reverse_runs_fused(const fdtd_handle* h) {
+  return fused_reverse(h) && !direct_reverse(h) &&
+         (h->opt_reverse == 2 || !direct_shape(h) || cells_of(h) >= kFusedReverseCells);
+}
+
 // The field buffer holding the state after a forward: the fused step flips
-// the pair every step, the two-step pass every pair of steps (and its split
-// first step, for an odd count, once).
+// the pair every step (a layout of one field buffer ends in it, see
+// enqueue_forward), the two-step pass every pair of steps (and its first step,
+// for an odd count, once).
 static int forward_end_buf(const fdtd_handle* h) {
-  if (direct_forward(h)) return 0;
-  if (two_step_forward(h)) return ((h->N + 1) / 2) & 1;
-  return fused_forward(h) ? (h->N & 1) : 0;
+  const ForwardForm f = forward_form(h);
+  if (f == kTwoStep) return ((h->N + 1) / 2) & 1;
+  const bool pair = fused_reverse(h) || fused_forward(h) || two_step_forward(h);
+  return f == kFusedStep && pair ? (h->N & 1) : 0;
 }
 
 // ---------------------------------------------------------------- layout ---
@@ -1267,7 +1299,8 @@ struct ZGroups {
 // Streams and events of the z-group scheduling of direction dir (created as
 // needed, outside a capture).
 static cudaError_t ensure_zgroups(fdtd_handle* h, int dir) {
-  const int want = zgroups_of(h, dir);
+  int want = zgroups_of(h, dir);
+  if (want > 1 && dir == 0 && forward_form(h) != kSplit) want = std::max(want, 3);
   if (want <= 1 || (int)h->zs.size() >= want) return cudaSuccess;
   cudaError_t e = cudaSuccess;
   if (!h->zfork) e = cudaEventCreateWithFlags(&h->zfork, cudaEventDisableTiming);
@@ -1333,7 +1366,7 @@ static cudaError_t enqueue_forward(fdtd_handle* h, const fdtd_record_cfg* rec, i
   if (det2.kind && (e = cudaMemsetAsync(h->ws + L.obj2, 0, h->N * sizeof(double), h->stream)))
     return e;
   Sampler smp(h, 0);
-  if (direct_forward(h)) {
+  if (forward_form(h) == kDirect) {
     // two launches per step; an unscaled record rides in them unless kernel
     // timing is being sampled (which times one kind per launch)
     DirectArgs d = direct_args(h, L, a);
@@ -1375,188 +1408,130 @@ static cudaError_t enqueue_forward(fdtd_handle* h, const fdtd_record_cfg* rec, i
     *launches = nl;
     return cudaSuccess;
   }
-  if (two_step_forward(h)) {
-    // two steps per pass: steps n, n + 1 of the deep units in one launch on
-    // the main stream (buffer cur -> cur ^ 1, the intermediate level's frame
-    // -> buffer 2), the split H half-step of step n over the other units
-    // beside it on a side stream (cur -> 2), then their split E half-step of
-    // step n (cur -> 2) and both half-steps of step n + 1 (2 -> cur ^ 1); the
-    // auxiliaries stay in place.  An odd count runs step 0 as split
-    // half-steps over every unit (cur -> cur ^ 1).
+  const ForwardForm form = forward_form(h);
+  if (form == kTwoStep || form == kFusedStep) {
+    // Fused forward steps (kernels_fwd_fused.cu): every unit of a step, or, with
+    // two steps per pass, the units outside the deep box.  Field buffers and
+    // auxiliary sets are read and written in turn.  With a layout of one field
+    // buffer the adjoint's, which the forward leaves idle, is the other one, and
+    // an odd count starts there, so that the run ends in buffer 0; likewise the
+    // first adjoint auxiliary set is the second forward set.
+    const bool two = form == kTwoStep;
     const int zcs = fused_forward_zchunk(h);
     a.zchunk = zcs;
-    const RevUnits D = deep_units(a.g, zcs);
-    RevUnits all = D;   // no deep box: the ring decode covers every unit
-    all.ix0 = all.ix1 = all.iy0 = all.iy1 = all.iz0 = all.iz1 = 0;
-    // planes per CTA of the pass: 16 split chunks by default (600 x 600 x 300,
-    // 1000-step runs: 1055, 1036 and 1028 us per forward step with 4, 8 and
-    // 16 chunks; each chunk re-reads two planes below and one above it)
-    const int zdeep = h->opt_zchunk_fwd2 > 0 ? h->opt_zchunk_fwd2 : 16 * zcs;
-    const float* Fb[3];
-    for (int b = 0; b < 3; ++b) Fb[b] = (const float*)(h->ws + L.F[b]);
+    const bool lent = L.F[1] == L.F[0];
+    const size_t fo[3] = {L.F[0], lent ? L.L[0] : L.F[1], L.F[2]};
+    const size_t po[2] = {L.psiF[0], L.psiL[0]};
+    const RevUnits D = two ? deep_units(a.g, zcs) : rev_units(a.g, zcs);
+    const RevUnits R = rev_units(a.g, zcs);
     const float* cbp = (const float*)(h->ws + L.cb);
-    const float* ps = (const float*)(h->ws + L.psiF[0]);
     Fwd2Maps dm[2];
-    LagMaps lh[3], le[3][3];   // le[i][o]: E of buffer i, Ht^{n+1/2} of buffer o
-    for (int b = 0; b < 3; ++b) {
-      if (b < 2 && (e = encode_fwd2_maps(Fb[b], cbp, a.g, &dm[b]))) return e;
-      if ((e = encode_lag_maps(Fb[b], Fb[b], cbp, ps, a.g, 8, 32, L.plF, &lh[b]))) return e;
-      for (int o = 0; o < 3; ++o)
-        if (o != b && (e = encode_lag_maps(Fb[b], Fb[b], cbp, ps, a.g, 8, 32, L.plF, &le[b][o],
-                                           Fb[o])))
+    FwdMaps fm[3][2];   // fields of buffer b, auxiliaries of set q
+    for (int b = 0; b < (two ? 3 : 2); ++b) {
+      const float* Fb = (const float*)(h->ws + fo[b]);
+      if (two && b < 2 && (e = encode_fwd2_maps(Fb, cbp, a.g, &dm[b]))) return e;
+      for (int q = 0; q < 2; ++q)
+        if ((e = encode_fwd_maps(Fb, cbp, (const float*)(h->ws + po[q]), a.g, L.plF, &fm[b][q])))
           return e;
     }
-    const bool conc = h->opt_sample == 0 && h->opt_zgroups != 1 && !h->zs.empty() &&
-                      h->zev.size() >= 3;
-    // one split time step over the units of U (umode 1 and 2) from buffer i
-    // into buffer o, with its record and second detector
-    auto split_step = [&](int n, int i, int o, const RevUnits& U, cudaStream_t hs,
-                          bool h_done) -> cudaError_t {
+    // planes per CTA of the two-step pass: 16 split chunks by default (600 x 600 x
+    // 300, us per forward step with 4, 8 and 16 chunks: 1055, 1036, 1028, with the
+    // split half-steps outside the deep box)
+    const int zdeep = h->opt_zchunk_fwd2 > 0 ? h->opt_zchunk_fwd2 : 16 * zcs;
+    const bool conc = h->opt_sample == 0 && h->opt_zgroups != 1 && h->zs.size() >= 3 &&
+                      h->zev.size() >= 9;
+    int cur = lent ? (h->N & 1) : 0, ps = 0;
+    if (cur == 1 && (e = cudaMemsetAsync(h->ws + fo[1], 0, nc6, h->stream))) return e;
+    // The launches of step n from buffer i into buffer o over the kinds [first, 5)
+    // of U's units, each kind on its own stream between a fork and a join when
+    // they may overlap.
+    auto fork = [&]() -> cudaError_t {
+      if (!conc) return cudaSuccess;
+      cudaError_t e2 = cudaEventRecord(h->zev[0], h->stream);
+      for (int t = 0; !e2 && t < 3; ++t) e2 = cudaStreamWaitEvent(h->zs[t], h->zev[0], 0);
+      return e2;
+    };
+    auto join = [&]() -> cudaError_t {
+      cudaError_t e2 = cudaSuccess;
+      for (int t = 0; conc && !e2 && t < 3; ++t) {
+        e2 = cudaEventRecord(h->zev[3 * t + 1], h->zs[t]);
+        if (!e2) e2 = cudaStreamWaitEvent(h->stream, h->zev[3 * t + 1], 0);
+      }
+      return e2;
+    };
+    auto units_step = [&](int n, int i, int o, const RevUnits& U, int first) -> cudaError_t {
       StepArgs b = a;
-      b.U = U;
-      b.zchunk = zcs;
       b.jn = h->wave[n];
       b.obj = (double*)(h->ws + L.obj) + n;
-      b.F = (float*)(h->ws + L.F[i]);
-      b.Fn = (float*)(h->ws + L.F[o]);
+      b.F = (float*)(h->ws + fo[i]);
+      b.Fn = (float*)(h->ws + fo[o]);
+      b.psiA = (float*)(h->ws + po[ps]);
+      b.psiB = (float*)(h->ws + po[ps ^ 1]);
       cudaError_t e2;
-      if (!h_done) {
-        if ((e2 = smp.before(FDTD_K_FWD_H))) return e2;
-        for (int um = 1; um <= 2; ++um) {
-          b.umode = um;
-          if ((e2 = launch_lag2(0, lh[i], b, hs))) return e2;
-        }
-        if ((e2 = smp.after(FDTD_K_FWD_H))) return e2;
-        nl += 2;
-        return cudaSuccess;
+      if ((e2 = smp.before(FDTD_K_FWD_FUSED))) return e2;
+      // the CPML-free units beside the others: main stream 0, sides 2, 3 + 4, 1
+      static const int kStream[5] = {-1, 2, 0, 1, 1};
+      for (int kind = 4; kind >= first; --kind) {
+        cudaStream_t st = conc && kStream[kind] >= 0 ? h->zs[kStream[kind]] : h->stream;
+        if ((e2 = launch_fwd_fused(kind, fm[i][ps], b, U, st))) return e2;
+        ++nl;
       }
-      if ((e2 = smp.before(FDTD_K_FWD_E))) return e2;
-      for (int um = 1; um <= 2; ++um) {
-        b.umode = um;
-        if ((e2 = launch_lag2(1, le[i][o], b, h->stream))) return e2;
-      }
-      if ((e2 = smp.after(FDTD_K_FWD_E))) return e2;
-      nl += 2;
-      const bool rec_now = n >= r && (n - r) % rec->k == 0;
-      if (rec_now) {   // E^n in buffer i, Ht^{n+1/2} in buffer o
+      if ((e2 = smp.after(FDTD_K_FWD_FUSED))) return e2;
+      ps ^= 1;
+      return cudaSuccess;
+    };
+    // the record and the second detector after step n (buffers i -> o)
+    auto after_step = [&](int n, int i, int o) -> cudaError_t {
+      cudaError_t e2;
+      if (n >= r && (n - r) % rec->k == 0) {   // E^n in buffer i, Ht^{n+1/2} in buffer o
         if ((e2 = smp.before(FDTD_K_RECORD))) return e2;
-        if ((e2 = record(b.Fn, b.F, (n - r) / rec->k))) return e2;
+        if ((e2 = record((const float*)(h->ws + fo[o]), (const float*)(h->ws + fo[i]),
+                         (n - r) / rec->k)))
+          return e2;
         if ((e2 = smp.after(FDTD_K_RECORD))) return e2;
         ++nl;
       }
       if (det2.kind) {
         if ((e2 = smp.before(FDTD_K_MONITOR))) return e2;
-        if ((e2 = launch_monitor(b.Fn, a.g, det2, (double*)(h->ws + L.obj2) + n, h->stream)))
+        if ((e2 = launch_monitor((const float*)(h->ws + fo[o]), a.g, det2,
+                                 (double*)(h->ws + L.obj2) + n, h->stream)))
           return e2;
         if ((e2 = smp.after(FDTD_K_MONITOR))) return e2;
         ++nl;
       }
       return cudaSuccess;
     };
-    int cur = 0, n = 0;
-    if (h->N & 1) {
-      if ((e = split_step(0, cur, cur ^ 1, all, h->stream, false))) return e;
-      if ((e = split_step(0, cur, cur ^ 1, all, h->stream, true))) return e;
+    int n = 0;
+    for (; n < (two ? (h->N & 1) : h->N); ++n) {   // one step over every unit
+      if ((e = fork())) return e;
+      if ((e = units_step(n, cur, cur ^ 1, R, 0))) return e;
+      if ((e = join())) return e;
+      if ((e = after_step(n, cur, cur ^ 1))) return e;
       cur ^= 1;
-      n = 1;
     }
+    // two steps per pass: steps n, n + 1 of the deep units in one launch (buffer
+    // cur -> cur ^ 1, the intermediate level's frame -> buffer 2) beside step n of
+    // the other units (cur -> 2), which reads nothing the pass writes; then their
+    // step n + 1 (2 -> cur ^ 1), which reads the frame
     for (; n + 1 < h->N; n += 2) {
-      cudaStream_t side = conc ? h->zs[0] : h->stream;
-      if (conc) {
-        if ((e = cudaEventRecord(h->zev[0], h->stream))) return e;
-        if ((e = cudaStreamWaitEvent(side, h->zev[0], 0))) return e;
-      }
       StepArgs b = a;
-      b.F = (float*)(h->ws + L.F[cur]);
-      b.Fn = (float*)(h->ws + L.F[cur ^ 1]);
-      b.Fm = (float*)(h->ws + L.F[2]);
+      b.F = (float*)(h->ws + fo[cur]);
+      b.Fn = (float*)(h->ws + fo[cur ^ 1]);
+      b.Fm = (float*)(h->ws + fo[2]);
       b.zcs = zcs;
       b.zchunk = zdeep;
+      if ((e = fork())) return e;
       if ((e = smp.before(FDTD_K_FWD_2STEP))) return e;
       if ((e = launch_fwd_2step(dm[cur], b, D, h->stream))) return e;
       if ((e = smp.after(FDTD_K_FWD_2STEP))) return e;
       ++nl;
-      if ((e = split_step(n, cur, 2, D, side, false))) return e;
-      if (conc) {
-        if ((e = cudaEventRecord(h->zev[1], side))) return e;
-        if ((e = cudaStreamWaitEvent(h->stream, h->zev[1], 0))) return e;
-      }
-      if ((e = split_step(n, cur, 2, D, h->stream, true))) return e;
-      if ((e = split_step(n + 1, 2, cur ^ 1, D, h->stream, false))) return e;
-      if ((e = split_step(n + 1, 2, cur ^ 1, D, h->stream, true))) return e;
-      cur ^= 1;
-    }
-    *launches = nl;
-    return cudaSuccess;
-  }
-  if (fused_forward(h)) {
-    // fused forward step: the CPML-free units in one launch on the main
-    // stream, the split H half-step of the other units beside it on a side
-    // stream, then their split E half-step; buffer cur of the fields is read
-    // and buffer cur ^ 1 written (the auxiliaries stay in place)
-    a.zchunk = fused_forward_zchunk(h);
-    const RevUnits U = rev_units(a.g, a.zchunk);
-    RevMaps fm[2];
-    LagMaps lh[2], le[2];
-    for (int b = 0; b < 2; ++b) {
-      const float* Fb = (const float*)(h->ws + L.F[b]);
-      const float* Fo = (const float*)(h->ws + L.F[b ^ 1]);
-      const float* cbp = (const float*)(h->ws + L.cb);
-      const float* ps = (const float*)(h->ws + L.psiF[0]);
-      if ((e = encode_rev_maps(Fb, Fb, cbp, ps, a.g, L.plF, &fm[b]))) return e;
-      if ((e = encode_lag_maps(Fb, Fb, cbp, ps, a.g, 8, 32, L.plF, &lh[b]))) return e;
-      if ((e = encode_lag_maps(Fb, Fb, cbp, ps, a.g, 8, 32, L.plF, &le[b], Fo))) return e;
-    }
-    const bool conc = h->opt_sample == 0 && h->opt_zgroups != 1 && !h->zs.empty() &&
-                      h->zev.size() >= 3;
-    int cur = 0;
-    for (int n = 0; n < h->N; ++n) {
-      a.jn = h->wave[n];
-      a.obj = (double*)(h->ws + L.obj) + n;
-      a.F = (float*)(h->ws + L.F[cur]);
-      a.Fn = (float*)(h->ws + L.F[cur ^ 1]);
-      const bool rec_now = n >= r && (n - r) % rec->k == 0;
-      const int j = rec_now ? (n - r) / rec->k : 0;
-      cudaStream_t side = conc ? h->zs[0] : h->stream;
-      if (conc) {
-        if ((e = cudaEventRecord(h->zev[0], h->stream))) return e;
-        if ((e = cudaStreamWaitEvent(side, h->zev[0], 0))) return e;
-      }
-      StepArgs b = a;
-      b.U = U;
-      if ((e = smp.before(FDTD_K_FWD_FUSED))) return e;
-      if ((e = launch_fwd_fused(fm[cur], a, U, h->stream))) return e;
-      if ((e = smp.after(FDTD_K_FWD_FUSED))) return e;
-      if ((e = smp.before(FDTD_K_FWD_H))) return e;
-      for (int um = 1; um <= 2; ++um) {
-        b.umode = um;
-        if ((e = launch_lag2(0, lh[cur], b, side))) return e;
-      }
-      if ((e = smp.after(FDTD_K_FWD_H))) return e;
-      if (conc) {
-        if ((e = cudaEventRecord(h->zev[1], side))) return e;
-        if ((e = cudaStreamWaitEvent(h->stream, h->zev[1], 0))) return e;
-      }
-      if ((e = smp.before(FDTD_K_FWD_E))) return e;
-      for (int um = 1; um <= 2; ++um) {
-        b.umode = um;
-        if ((e = launch_lag2(1, le[cur], b, h->stream))) return e;
-      }
-      if ((e = smp.after(FDTD_K_FWD_E))) return e;
-      nl += 5;
-      if (rec_now) {   // E^n is still in buffer cur, Ht^{n+1/2} now in cur ^ 1
-        if ((e = smp.before(FDTD_K_RECORD))) return e;
-        if ((e = record(a.Fn, a.F, j))) return e;
-        if ((e = smp.after(FDTD_K_RECORD))) return e;
-        ++nl;
-      }
-      if (det2.kind) {
-        if ((e = smp.before(FDTD_K_MONITOR))) return e;
-        if ((e = launch_monitor(a.Fn, a.g, det2, (double*)(h->ws + L.obj2) + n, h->stream)))
-          return e;
-        if ((e = smp.after(FDTD_K_MONITOR))) return e;
-        ++nl;
-      }
+      if ((e = units_step(n, cur, 2, D, 1))) return e;
+      if ((e = join())) return e;
+      if ((e = after_step(n, cur, 2))) return e;
+      if ((e = fork())) return e;
+      if ((e = units_step(n + 1, 2, cur ^ 1, D, 1))) return e;
+      if ((e = join())) return e;
+      if ((e = after_step(n + 1, 2, cur ^ 1))) return e;
       cur ^= 1;
     }
     *launches = nl;
@@ -1625,7 +1600,7 @@ static cudaError_t enqueue_backward(fdtd_handle* h, const fdtd_record_cfg* rec, 
   int nl = 0;
   // the adjoint starts at zero in the buffer the first step reads: the fused
   // reverse step starts in the forward's buffer, the split phases work in 0
-  const bool direct = direct_reverse(h), fused = !direct && fused_reverse(h);
+  const bool direct = direct_reverse(h), fused = reverse_runs_fused(h);
   const int lam0 = fused ? h->fwd_buf : 0;
   if ((e = cudaMemsetAsync(h->ws + L.L[lam0], 0, nc6, h->stream))) return e;
   if ((e = cudaMemsetAsync(h->ws + L.psiL[0], 0, psb, h->stream))) return e;
@@ -2010,7 +1985,7 @@ static int backward_async(fdtd_handle* h, double seed, double seed2) {
   h->have_forward = false;
   // the fused reverse step leaves the reconstructed fields in the buffer of
   // the last step's output
-  if (!direct_reverse(h) && fused_reverse(h)) h->fwd_buf ^= h->N & 1;
+  if (reverse_runs_fused(h)) h->fwd_buf ^= h->N & 1;
   return FDTD_OK;
 }
 

@@ -287,8 +287,7 @@ struct StepArgs {
   float* psiA;     // psi set read (and written in place by the forward)
   float* psiB;     // psi set written (ping-pong)
   float* L;        // adjoint fields (6 components, same layout as F)
-  float* Fn;       // fused steps: fields written (the other buffer of a ping-pong pair);
-                   // the forward half-steps write here when set, else in place
+  float* Fn;       // fused steps: fields written (the other buffer of a ping-pong pair)
   float* Ln;       // fused reverse step: adjoint fields written
   float* Fm;       // two-step forward: the intermediate time level (frame of the deep box)
   double* gacc;    // FP64 design-box accumulator [dz][dy][dx]
@@ -301,8 +300,6 @@ struct StepArgs {
   int zc0, zc1;     // two-cells-per-thread kernels: z chunks [zc0, zc1) of this launch (zc1 = 0: to the last)
   int zcs;          // two-step forward: planes per z chunk of U (the split half-steps' chunks)
   int t0x, t0y;     // fused reverse step: first tile of a launch along x and y
-  int umode;        // forward half-steps (32 x 8 tiles): 0 every unit of the grid (offset
-                    // by zc0), 1 the z-only units of U, 2 the ring units of U
   RevUnits U;
   // batched designs (the BM kernel instantiations): CTA b runs unit bunits[b]
   // = (design, tile x, tile y, z chunk) of design bargs[design] (that
@@ -331,11 +328,8 @@ cudaError_t launch_fwd_e(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_rev_e(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_rev_h(const StepArgs& a, cudaStream_t s);
 
-// Fwide (optional): the field buffer of the wide boxes Fw (the forward E
-// half-step of a fused forward reads Ht^{n+1/2} from the buffer being written).
 cudaError_t encode_lag_maps(const float* F, const float* L, const float* cb, const float* psiA,
-                            const Geo& g, int ty, int tw, const PsiLayout& pl, LagMaps* m,
-                            const float* Fwide = nullptr);
+                            const Geo& g, int ty, int tw, const PsiLayout& pl, LagMaps* m);
 // Staged half-steps, two x-cells per thread (kernel 5; tile height >= 2).
 // which: 0 forward H, 1 forward E, 2 reverse E phase, 3 reverse H phase.
 cudaError_t launch_lag2(int which, const LagMaps& m, const StepArgs& a, cudaStream_t s);
@@ -368,15 +362,24 @@ long long rev_ring_tiles(const RevUnits& U);
 // Reads a.F, a.L, a.psiA; writes a.Fn, a.Ln, a.psiB, a.gacc.
 cudaError_t launch_rev_fused(int which, const RevMaps& m, const StepArgs& a, const RevUnits& U,
                              cudaStream_t s);
-// The fused forward step (kernels_fwd_fused.cu) over the units [ix0, ix1) x
-// [iy0, iy1) x [iz0, iz1) of U (none may hold a source or detector cell):
-// reads a.F (E^n, Ht^{n-1/2}) and cb, writes a.Fn (E^{n+1}, Ht^{n+1/2}).
-cudaError_t launch_fwd_fused(const RevMaps& m, const StepArgs& a, const RevUnits& U,
+// The fused forward step (kernels_fwd_fused.cu): tensor maps over the fields and
+// the auxiliaries of the set read (boxes: F40 40 x 10 and F36 36 x 9, 3 components;
+// cb32 32 x 8; Qx36, Qy36, Qz36 36 x 9, Qxo, Qyo, Qzo 32 x 8, 2 components).
+struct alignas(64) FwdMaps {
+  CUtensorMap F40, F36, cb32, Qx36, Qy36, Qz36, Qxo, Qyo, Qzo;
+};
+cudaError_t encode_fwd_maps(const float* F, const float* cb, const float* psiA, const Geo& g,
+                            const PsiLayout& pl, FwdMaps* m);
+// kind: 0 the units [ix0, ix1) x [iy0, iy1) x [iz0, iz1) of U, 1 the other chunks of
+// those tiles, 2 the tile columns beside them, 3 the tile rows beside them, 4 the
+// corners (2-4: every chunk).  Reads a.F (E^n, Ht^{n-1/2}), cb and the auxiliaries
+// the maps view, writes a.Fn (E^{n+1}, Ht^{n+1/2}) and a.psiB.
+cudaError_t launch_fwd_fused(int kind, const FwdMaps& m, const StepArgs& a, const RevUnits& U,
                              cudaStream_t s);
 // Two forward time steps per pass (kernels_fwd_2step.cu): tensor maps over
-// the fields (boxes 40 x 12, 3 components) and cb (40 x 10).
+// the fields (boxes 40 x 20, 3 components) and cb (40 x 18).
 struct alignas(64) Fwd2Maps {
-  CUtensorMap F4012, cb40;
+  CUtensorMap F40, cb40;
 };
 cudaError_t encode_fwd2_maps(const float* F, const float* cb, const Geo& g, Fwd2Maps* m);
 // The deep units of a grid for split z chunks of zcs planes: the tiles and

@@ -9,13 +9,13 @@
 // A CTA reads E^n, Ht^{n-1/2} and cb of its unit once and writes E2 and Ht2
 // once (52 B per cell for two time steps, against 104 B for two fused
 // steps).  The intermediate level exists only in shared memory, on halos
-// that shrink by one cell per half-step: E2 on the 32 x 8 tile T needs Ht2
+// that shrink by one cell per half-step: E2 on the 32 x 16 tile T needs Ht2
 // on T and its -x / -y neighbours (R1), Ht2 on R1 needs E1 on R1 and its
 // +x / +y neighbours (R2), E1 on R2 needs Ht1 on R2 and its -x / -y
 // neighbours (R3), and Ht1 on R3 needs E^n on R3 and its +x / +y neighbours
 // (R4).  One thread per pair of x cells on R3: 18 pair columns (x = x0 - 2 +
-// 2 px) by 11 rows (y = y0 - 2 + ry); R2 is rows ry >= 1, R1 rows 1..9 and
-// pair columns 0..16, T rows 2..9 and pair columns 1..16.  Along z the
+// 2 px) by 19 rows (y = y0 - 2 + ry); R2 is rows ry >= 1, R1 rows 1..17 and
+// pair columns 0..16, T rows 2..17 and pair columns 1..16.  Along z the
 // levels lag one plane each: with E^n of plane p staged, the CTA finishes
 // Ht1(p - 1), updates E1(p - 1), then Ht2(p - 2) and E2(p - 2); a chunk
 // [k0, k1) streams the planes k0 - 2 .. k1 + 1.
@@ -23,12 +23,22 @@
 // The launch covers the deep units: every cell on which the CTA evaluates a
 // level (R3 over the planes k0 - 2 .. k1) lies in the interior, so no CPML
 // term arises, and the host keeps the source and the detectors away from
-// them.  The other units run the split half-steps one time step at a time,
-// through a third buffer Fm that holds the intermediate level: they need
-// E1 and Ht1 only on the deep units' cells next to their own, i.e. on the
-// one-cell frame of the deep box, which this kernel writes into Fm.  Every
-// cell sees the same explicitly rounded operations as in the split and the
-// fused kernels, so the fields are bit-identical to theirs.
+// them.  The other units run the fused step one time step at a time, through a
+// third buffer Fm that holds the intermediate level: they need E1 and Ht1 only
+// on the deep units' cells next to their own, i.e. on the one-cell frame of the
+// deep box, which this kernel writes into Fm.  Every cell sees the same
+// explicitly rounded operations as in the split and the fused kernels, so the
+// fields are bit-identical to theirs.
+//
+// What bounds it: latency, at 22 warps per SM and 0.4 instructions per cycle and
+// scheduler (DRAM at half its rate).  The tile is 16 rows high because the halo
+// work falls with it: 1.34 pair tasks a useful one against 1.55 at 8 rows (us per
+// forward step on 600 x 600 x 300, with the fused step outside the deep box: 962 at 8
+// rows and three CTAs per SM, 916 at 16 and two, 961 at 32 and one); two block
+// barriers per plane instead of three: 907; E1 of the pair's own cells from
+// registers instead of shared memory: 888.  Not faster: two stages (933), one barrier
+// per plane with double level arrays (1046 against 1031 at 8 rows: the stages are
+// refilled later), FP32 pairs in packed instructions (887).
 #include <cudaTypedefs.h>
 
 #include "lag_common.cuh"
@@ -39,20 +49,21 @@ using namespace lag2;
 
 namespace fwd2s {
 
-constexpr int TW = 32, TY = 8;
-constexpr int NPX = 18, NRY = 11, NT = NPX * NRY;   // pair tasks of R3
-constexpr int THREADS = 224;                        // 7 warps
+constexpr int TW = 32, TY = 16;                     // tile of a CTA
+constexpr int UY = 8;                               // rows of a unit (the deep box's granularity)
+constexpr int NPX = 18, NRY = TY + 3, NT = NPX * NRY;   // pair tasks of R3
+constexpr int THREADS = (NT + 31) / 32 * 32;
 constexpr int BW = 40;                              // row width: x in [x0 - 4, x0 + 36)
 
 // Shared memory (byte offsets): S stages of an E^n box and an Ht^{n-1/2}
-// box, 40 x 12 at (x0 - 4, y0 - 2), 3 components each, and a cb box 40 x 10
+// box, 40 x 20 at (x0 - 4, y0 - 2), 3 components each, and a cb box 40 x 18
 // at (x0 - 4, y0 - 1); the stages' mbarriers after them; then Ht1 of one
 // plane, E1 of two planes (ping-pong by plane parity) and Ht2 of one plane,
-// each [3][11][40] at (x0 - 4, y0 - 2).
+// each [3][19][40] at (x0 - 4, y0 - 2).
 template <int S>
 struct L2S {
-  static constexpr int BP = BW * 12;    // one component of a staged field box
-  static constexpr int CBP = BW * 10;   // the cb box
+  static constexpr int BP = BW * (TY + 4);    // one component of a staged field box
+  static constexpr int CBP = BW * (TY + 2);   // the cb box
   static constexpr int AP = BW * NRY;   // one component of a level's plane array
   static constexpr int E = 0;
   static constexpr int H = E + r128(3 * BP * 4);
@@ -69,23 +80,23 @@ static_assert(L2S<3>::H1 >= L2S<3>::BARS + 8 * 3, "level arrays after the barrie
 static_assert(NT <= THREADS, "one pair task per thread");
 
 template <int S, bool EX>
-__global__ void __launch_bounds__(THREADS, 3)
+__global__ void __launch_bounds__(THREADS, 2)
 k_fwd_2step(const __grid_constant__ Fwd2Maps m, StepArgs a) {
   typedef L2S<S> Y;
   extern __shared__ __align__(128) unsigned char dsm[];
   const Geo& g = a.g;
   const int tid = threadIdx.x;
-  const int x0 = (blockIdx.x + a.U.ix0) * TW, y0 = (blockIdx.y + a.U.iy0) * TY;
+  const int x0 = (blockIdx.x + a.U.ix0) * TW, y0 = a.U.iy0 * UY + blockIdx.y * TY;
   // the deep box in cells, and this CTA's chunk of it
-  const int X0 = a.U.ix0 * TW, X1 = a.U.ix1 * TW, Y0 = a.U.iy0 * TY, Y1 = a.U.iy1 * TY;
+  const int X0 = a.U.ix0 * TW, X1 = a.U.ix1 * TW, Y0 = a.U.iy0 * UY, Y1 = a.U.iy1 * UY;
   const int Z0 = a.U.iz0 * a.zcs, Z1 = min(g.nz, a.U.iz1 * a.zcs);
   const int k0 = Z0 + blockIdx.z * a.zchunk, k1 = min(Z1, k0 + a.zchunk);
   const bool task = tid < NT;
   const int px = task ? tid % NPX : 0, ry = task ? tid / NPX : 0;
   const int x = x0 - 2 + 2 * px, y = y0 - 2 + ry;
   const bool r2 = task && ry >= 1;                         // R2
-  const bool r1 = r2 && ry <= 9 && px <= 16;               // R1
-  const bool tt = r1 && ry >= 2 && px >= 1;                // T
+  const bool r1 = r2 && ry <= TY + 1 && px <= 16;               // R1
+  const bool tt = r1 && ry >= 2 && px >= 1 && y < Y1;                // T
   const int hb = ry * BW + (x - x0 + 4);                   // the pair in a box or level array
   const int cbi = (ry - 1) * BW + (x - x0 + 4);            // the pair in the cb box (R2)
   // frame cells of the deep box (the intermediate level goes to Fm there)
@@ -94,8 +105,8 @@ k_fwd_2step(const __grid_constant__ Fwd2Maps m, StepArgs a) {
   const int p0_ = k0 - 2, p1_ = k1 + 1;
   uint64_t* bars = ring_init<S>(dsm, Y::STAGE);   // at Y::BARS
   auto boxes = [&](int p, auto&& f) {
-    f(Y::E, &m.F4012, x0 - 4, y0 - 2, p, 0, 3 * Y::BP * 4);
-    if (p <= k1) f(Y::H, &m.F4012, x0 - 4, y0 - 2, p, 3, 3 * Y::BP * 4);
+    f(Y::E, &m.F40, x0 - 4, y0 - 2, p, 0, 3 * Y::BP * 4);
+    if (p <= k1) f(Y::H, &m.F40, x0 - 4, y0 - 2, p, 3, 3 * Y::BP * 4);
     if (p >= k0 - 1 && p <= k1) f(Y::CB, &m.cb40, x0 - 4, y0 - 1, p, 0, Y::CBP * 4);
   };
   auto issue = [&](int p, unsigned char* st, uint64_t* bar) {
@@ -129,7 +140,6 @@ k_fwd_2step(const __grid_constant__ Fwd2Maps m, StepArgs a) {
   for (int p = p0_; p <= p1_; ++p) {
     unsigned char* st = dsm + stg * Y::STAGE;
     if (!mbar_wait(bars + stg, par, kWaitCycles)) ok = false;
-    if (!__syncthreads_and(ok)) { ring_abort<S>(bars, stg, par, p, p1_, a.err); return; }
     const float* Eb = reinterpret_cast<const float*>(st + Y::E);
     // ---- A: finish Ht1(p - 1) with dEy/dz and dEx/dz ----
     float fx[2] = {0.f, 0.f}, fy[2] = {0.f, 0.f}, fz[2] = {0.f, 0.f};
@@ -159,7 +169,8 @@ k_fwd_2step(const __grid_constant__ Fwd2Maps m, StepArgs a) {
         }
       }
     }
-    __syncthreads();   // Ht1(p - 1) of R3 is in SH1
+    // Ht1(p - 1) of R3 is in SH1; a wait that gave up ends the CTA here
+    if (!__syncthreads_and(ok)) { ring_abort<S>(bars, stg, par, p, p1_, a.err); return; }
     // ---- B1: E1(p - 1) on R2 ----
     float ux[2] = {0.f, 0.f}, uy[2] = {0.f, 0.f}, uz[2] = {0.f, 0.f};   // E1(p - 1)
     const bool b1 = r2 && p >= k0 && p <= k1 + 1;
@@ -199,7 +210,8 @@ k_fwd_2step(const __grid_constant__ Fwd2Maps m, StepArgs a) {
     float gx[2] = {0.f, 0.f}, gy[2] = {0.f, 0.f}, gz[2] = {0.f, 0.f};   // Ht2(p - 2)
     if (r1 && p >= k0 + 1 && p <= k1 + 1) {
       const float* E1r = SE1 + (p & 1) * SE1P;   // plane p - 2
-      const float2 ex2 = ld2(E1r, hb), ey2 = ld2(E1r + AP, hb), ez2 = ld2(E1r + 2 * AP, hb);
+      const float2 ex2 = make_float2(c_e1x[0], c_e1x[1]), ey2 = make_float2(c_e1y[0], c_e1y[1]);
+      const float2 ez2 = make_float2(c_e1z[0], c_e1z[1]);
       const float2 ezy = ld2(E1r + 2 * AP, hb + BW), exy = ld2(E1r, hb + BW);   // +y
       const float ezx = E1r[2 * AP + hb + 2], eyx = E1r[AP + hb + 2];           // +x of cell 1
       const float t0[2] = {ezy.x - ez2.x, ezy.y - ez2.y};   // dEz/dy
@@ -305,8 +317,8 @@ RevUnits deep_units(const Geo& g, int zcs) {
   // x: R3 spans [x0 - 2, x0 + 34); y: [y0 - 2, y0 + 9); z: planes k0 - 2 .. k1
   U.ix0 = up(P + 2, TW);
   U.ix1 = g.nx - P - 34 >= 0 ? (g.nx - P - 34) / TW + 1 : 0;
-  U.iy0 = up(P + 2, TY);
-  U.iy1 = g.ny - P - 9 >= 0 ? (g.ny - P - 9) / TY + 1 : 0;
+  U.iy0 = up(P + 2, UY);
+  U.iy1 = g.ny - P - 9 >= 0 ? (g.ny - P - 9) / UY + 1 : 0;
   U.iz0 = up(P + 2, zc);
   U.iz1 = (g.nz - P - 1) / zc;   // full chunks ending at or below nz - P - 1
   if (U.ix1 <= U.ix0 || U.iy1 <= U.iy0 || U.iz1 <= U.iz0 || g.nx - 2 * P <= 0 ||
@@ -321,7 +333,7 @@ cudaError_t launch_fwd_2step(const Fwd2Maps& m, const StepArgs& a, const RevUnit
   if (!a.Fn || !a.Fm || a.zcs <= 0 || a.zchunk <= 0) return cudaErrorInvalidValue;
   if (U.ix1 <= U.ix0 || U.iy1 <= U.iy0 || U.iz1 <= U.iz0) return cudaSuccess;
   const int Z0 = U.iz0 * a.zcs, Z1 = U.iz1 * a.zcs < a.g.nz ? U.iz1 * a.zcs : a.g.nz;
-  const dim3 grid(U.ix1 - U.ix0, U.iy1 - U.iy0, (Z1 - Z0 + a.zchunk - 1) / a.zchunk);
+  const dim3 grid(U.ix1 - U.ix0, ((U.iy1 - U.iy0) * UY + TY - 1) / TY, (Z1 - Z0 + a.zchunk - 1) / a.zchunk);
   StepArgs b = a;
   b.U = U;
   const dim3 block(THREADS);

@@ -55,8 +55,7 @@ static cudaError_t enc_axis(CUtensorMap* m, const float* set, const PsiAxis& A, 
 }
 
 cudaError_t encode_lag_maps(const float* F, const float* Lm, const float* cb, const float* psiA,
-                            const Geo& g, int ty, int tw, const PsiLayout& pl, LagMaps* m,
-                            const float* Fwide) {
+                            const Geo& g, int ty, int tw, const PsiLayout& pl, LagMaps* m) {
   *m = LagMaps{};
   cudaError_t e;
   const int w = tw + 4;
@@ -65,7 +64,7 @@ cudaError_t encode_lag_maps(const float* F, const float* Lm, const float* cb, co
   if ((e = enc_axis(&m->Qyo, psiA, pl.ax[1], tw, ty))) return e;
   if ((e = enc_axis(&m->Qyw, psiA, pl.ax[1], tw, ty + 1))) return e;
   if ((e = enc_axis(&m->Qzo, psiA, pl.ax[2], tw, ty))) return e;
-  if ((e = enc3(&m->Fw, Fwide ? Fwide : F, g, 6, w, ty + 1, 3))) return e;
+  if ((e = enc3(&m->Fw, F, g, 6, w, ty + 1, 3))) return e;
   if ((e = enc3(&m->Fo, F, g, 6, tw, ty, 3))) return e;
   if ((e = enc3(&m->Lw, Lm, g, 6, w, ty + 1, 3))) return e;
   if ((e = enc3(&m->Lo, Lm, g, 6, tw, ty, 3))) return e;
@@ -94,11 +93,27 @@ cudaError_t encode_rev_maps(const float* F, const float* Lm, const float* cb, co
   return enc_axis(&m->Qzo, psiA, pl.ax[2], tw, ty);
 }
 
+cudaError_t encode_fwd_maps(const float* F, const float* cb, const float* psiA, const Geo& g,
+                            const PsiLayout& pl, FwdMaps* m) {
+  const int tw = 32, ty = 8;
+  *m = FwdMaps{};
+  cudaError_t e;
+  if ((e = enc3(&m->F40, F, g, 6, tw + 8, ty + 2, 3))) return e;
+  if ((e = enc3(&m->F36, F, g, 6, tw + 4, ty + 1, 3))) return e;
+  if ((e = enc3(&m->cb32, cb, g, 1, tw, ty, 1))) return e;
+  if ((e = enc_axis(&m->Qx36, psiA, pl.ax[0], tw + 4, ty + 1))) return e;
+  if ((e = enc_axis(&m->Qy36, psiA, pl.ax[1], tw + 4, ty + 1))) return e;
+  if ((e = enc_axis(&m->Qz36, psiA, pl.ax[2], tw + 4, ty + 1))) return e;
+  if ((e = enc_axis(&m->Qxo, psiA, pl.ax[0], tw, ty))) return e;
+  if ((e = enc_axis(&m->Qyo, psiA, pl.ax[1], tw, ty))) return e;
+  return enc_axis(&m->Qzo, psiA, pl.ax[2], tw, ty);
+}
+
 cudaError_t encode_fwd2_maps(const float* F, const float* cb, const Geo& g, Fwd2Maps* m) {
   *m = Fwd2Maps{};
   cudaError_t e;
-  if ((e = enc3(&m->F4012, F, g, 6, 40, 12, 3))) return e;
-  return enc3(&m->cb40, cb, g, 1, 40, 10, 1);
+  if ((e = enc3(&m->F40, F, g, 6, 40, 20, 3))) return e;
+  return enc3(&m->cb40, cb, g, 1, 40, 18, 1);
 }
 
 }  // namespace fdtd
