@@ -310,10 +310,10 @@ enum {
                                    as fdtd_selftest_wait */
   FDTD_OPT_REVERSE = 15,        /* kernel 5: how a reverse time step runs.  0 (default) =
                                    automatic: small grids the direct half-steps (as in
-                                   FDTD_OPT_FORWARD); from 9 million cells on fused with
-                                   32 x 8 tiles when at most half of the (tile, z chunk)
-                                   units carry CPML terms (see fdtd_reverse_units), else
-                                   split; 1 = split:
+                                   FDTD_OPT_FORWARD); larger ones fused with 32 x 8 tiles
+                                   when at most half of the (tile, z chunk) units carry
+                                   CPML terms (see fdtd_reverse_units), else split; 1 =
+                                   split:
                                    a reverse E phase and a reverse H phase, each updating the
                                    primal and the adjoint fields in place; 2 = fused: one
                                    launch for the primal fields (both inverse half-steps,

@@ -529,12 +529,13 @@ static bool direct_reverse(const fdtd_handle* h) {
 // else the fused step, and the fused reverse step where it may (fused_reverse).  us
 // per step, forward split / fused / two steps: 60 / 73 / 85 on 200 x 200 x 100 (4 M
 // cells), 127 / 132 / 141 on 301 x 203 x 151 (9.2 M), 144 / 147 / 133 on 300 x 300 x
-// 120 (10.8 M), 176 / 175 / 155 on 300 x 300 x 150 (13.5 M), 407 / - / 324 on 411 x
-// 389 x 203 (32 M); reverse split / fused: 104 / 120 (4 M), 195 / 199 (7.8 M), 224 /
-// 220 (9.2 M), 320 / 313 (13.5 M), 725 / 638 (32 M).  An option that names another
-// shape of the split half-steps leaves the choice to the units' CPML share alone.
+// 120 (10.8 M), 176 / 175 / 153 on 300 x 300 x 150 (13.5 M), 406 / - / 315 on 411 x
+// 389 x 203 (32 M); reverse split / fused: 95 / 89 on 180 x 180 x 100, 158 / 150 on
+// 200 x 200 x 150, 224 / 200 (9.2 M), 319 / 287 (13.5 M), 717 / 611 (32 M).  An
+// option that names another shape of the split half-steps leaves the choice to the
+// units' CPML share alone.
 enum ForwardForm { kSplit, kDirect, kFusedStep, kTwoStep };
-static const long long kFusedForwardCells = 12000000, kFusedReverseCells = 9000000;
+static const long long kFusedForwardCells = 12000000;
 static long long cells_of(const fdtd_handle* h) { return (long long)h->nx * h->ny * h->nz; }
 static ForwardForm forward_form(const fdtd_handle* h) {
   if (h->opt_kernel != 5 || h->opt_forward == 1) return kSplit;
@@ -547,8 +548,7 @@ static ForwardForm forward_form(const fdtd_handle* h) {
                                                                                      : kSplit;
 }
 static bool reverse_runs_fused(const fdtd_handle* h) {
-  return fused_reverse(h) && !direct_reverse(h) &&
-         (h->opt_reverse == 2 || !direct_shape(h) || cells_of(h) >= kFusedReverseCells);
+  return fused_reverse(h) && !direct_reverse(h);
 }
 
 // The field buffer holding the state after a forward: the fused step flips
@@ -1630,8 +1630,8 @@ static cudaError_t enqueue_backward(fdtd_handle* h, const fdtd_record_cfg* rec, 
   const RevUnits U = rev_units(a.g, a.zchunk);
   // the adjoint launches run on a side stream unless kernel timing is being
   // sampled or one launch per half-step is asked for (FDTD_OPT_ZGROUPS = 1)
-  const bool conc = fused && h->opt_sample == 0 && h->opt_zgroups != 1 && !h->zs.empty() &&
-                    h->zev.size() >= 3;
+  const bool conc = fused && h->opt_sample == 0 && h->opt_zgroups != 1 && h->zs.size() >= 3 &&
+                    h->zev.size() >= 9;
   for (int b = 0; fused && b < 2; ++b)
     if ((e = encode_rev_maps((const float*)(h->ws + L.F[b]), (const float*)(h->ws + L.L[b]),
                              (const float*)(h->ws + L.cb), (const float*)(h->ws + L.psiL[b]), a.g,
@@ -1719,27 +1719,34 @@ static cudaError_t enqueue_backward(fdtd_handle* h, const fdtd_record_cfg* rec, 
     a.psiA = (float*)(h->ws + L.psiL[cur]);
     a.psiB = (float*)(h->ws + L.psiL[cur ^ 1]);
     if (fused) {
-      // the primal and the adjoint launches of a step are independent: with
-      // a side stream the adjoint runs beside the primal, and the next
-      // step's restore waits for both
-      cudaStream_t side = conc ? h->zs[0] : h->stream;
+      // the primal and the three adjoint launches of a step are independent:
+      // each on its own stream, the heaviest units first, so that one launch's
+      // last CTAs leave room to the next (against one side stream for the three,
+      // us per reverse step: 600 x 600 x 300 1971 -> 1956, 411 x 389 x 203 637 -> 613,
+      // 301 x 203 x 151 220 -> 200); the next step's restore waits for all
+      cudaStream_t sd[3] = {h->stream, h->stream, h->stream};
       if (conc) {
         if ((e = cudaEventRecord(h->zev[0], h->stream))) return e;
-        if ((e = cudaStreamWaitEvent(side, h->zev[0], 0))) return e;
+        for (int t = 0; t < 3; ++t) {
+          sd[t] = h->zs[t];
+          if ((e = cudaStreamWaitEvent(sd[t], h->zev[0], 0))) return e;
+        }
       }
+      if ((e = smp.before(FDTD_K_REV_ADJOINT_CPML))) return e;
+      if ((e = launch_rev_fused(3, rmaps[cur], a, U, sd[2]))) return e;
+      if ((e = launch_rev_fused(2, rmaps[cur], a, U, sd[1]))) return e;
+      if ((e = smp.after(FDTD_K_REV_ADJOINT_CPML))) return e;
       if ((e = smp.before(FDTD_K_REV_PRIMAL))) return e;
       if ((e = launch_rev_fused(0, rmaps[cur], a, U, h->stream))) return e;
       if ((e = smp.after(FDTD_K_REV_PRIMAL))) return e;
       if ((e = smp.before(FDTD_K_REV_ADJOINT))) return e;
-      if ((e = launch_rev_fused(1, rmaps[cur], a, U, side))) return e;
+      if ((e = launch_rev_fused(1, rmaps[cur], a, U, sd[0]))) return e;
       if ((e = smp.after(FDTD_K_REV_ADJOINT))) return e;
-      if ((e = smp.before(FDTD_K_REV_ADJOINT_CPML))) return e;
-      if ((e = launch_rev_fused(2, rmaps[cur], a, U, side))) return e;
-      if ((e = launch_rev_fused(3, rmaps[cur], a, U, side))) return e;
-      if ((e = smp.after(FDTD_K_REV_ADJOINT_CPML))) return e;
       if (conc) {
-        if ((e = cudaEventRecord(h->zev[1], side))) return e;
-        if ((e = cudaStreamWaitEvent(h->stream, h->zev[1], 0))) return e;
+        for (int t = 0; t < 3; ++t) {
+          if ((e = cudaEventRecord(h->zev[3 * t + 1], sd[t]))) return e;
+          if ((e = cudaStreamWaitEvent(h->stream, h->zev[3 * t + 1], 0))) return e;
+        }
       }
       cur ^= 1;
       nl += 5;
