@@ -500,12 +500,12 @@ static bool two_step_forward(const fdtd_handle* h) {
 
 // Small grids run the direct half-steps (kernels_direct.cu) unless an option
 // names another form or shape.  The lines lie where they stop being faster
-// than the split staged ones (us per step, direct against split): forward
-// 5.2 / 26.7 at 0.11 M cells, 16.1 / 30.5 at 1.2 M, 23.6 / 35.1 at 1.8 M, 35.3 /
-// 38.5 at 2.6 M, 50.5 / 50.1 at 3.2 M, 63.5 / 60.1 at 4 M; reverse 6.9 / 30.6 at
-// 0.11 M, 27.6 / 39.0 at 1.2 M, 53.0 / 57.2 at 1.8 M, 78 / 73 at 2.6 M, 120 / 104 at
-// 4 M (beyond the L2 cache its re-read neighbour planes come from HBM).
-static const long long kDirectForwardCells = 3000000, kDirectReverseCells = 2000000;
+// than the split staged ones (us per step, direct against split): forward 4.9 / 26.7
+// at 0.11 M cells, 14.5 / 30.5 at 1.2 M, 25.5 / 34.6 at 2.1 M, 38.2 / 43.8 at 2.9 M,
+// 50.6 / 50.5 at 3.4 M; reverse 6.7 / 30.6 at 0.11 M, 27.4 / 39.0 at 1.2 M, 51.8 / 56.7 at
+// 1.8 M, 64.6 / 60.4 at 2.1 M, 118 / 104 at 4 M (beyond the L2 cache its re-read
+// neighbour planes come from HBM).
+static const long long kDirectForwardCells = 3400000, kDirectReverseCells = 2000000;
 static bool direct_shape(const fdtd_handle* h) {
   return h->opt_kernel == 5 && h->opt_tile_y == 8 && h->opt_tile_x == 32 && h->opt_stages == 2 &&
          h->opt_zchunk == 8 && h->opt_zchunk_fwd == -1 && h->opt_zgroups <= 1 && !h->opt_pdl &&
@@ -1898,15 +1898,22 @@ static int check_kernel_options(fdtd_handle* h) {
   return FDTD_OK;
 }
 
-static int forward_async(fdtd_handle* h, const float* d_eps, const fdtd_record_cfg* rec) {
+static int forward_check(fdtd_handle* h, const float* d_eps, const fdtd_record_cfg* rec) {
   int rc = check_rec(h, rec);
   if (rc) return rc;
   if (!d_eps) return fail(h, FDTD_EINVAL, "eps is NULL");
   rc = check_kernel_options(h);
   if (rc) return rc;
-  Layout L = layout_of(h, rec);
   if (!h->ws) return fail(h, FDTD_ESTATE, "no workspace bound");
-  if (L.total > h->ws_bytes) return fail(h, FDTD_ENOMEM, "workspace too small for this record config");
+  if (layout_of(h, rec).total > h->ws_bytes)
+    return fail(h, FDTD_ENOMEM, "workspace too small for this record config");
+  return FDTD_OK;
+}
+
+static int forward_async(fdtd_handle* h, const float* d_eps, const fdtd_record_cfg* rec) {
+  int rc = forward_check(h, d_eps, rec);
+  if (rc) return rc;
+  Layout L = layout_of(h, rec);
   rc = begin(h);
   if (rc) return rc;
   h->have_forward = false;
@@ -1976,11 +1983,17 @@ static cudaError_t upload_seeds(fdtd_handle* h, const Layout& L, double seed, do
   return cudaMemcpyAsync(h->ws + L.seeds, h->seeds, 2 * sizeof(double), cudaMemcpyHostToDevice, s);
 }
 
-static int backward_async(fdtd_handle* h, double seed, double seed2) {
+static int backward_check(fdtd_handle* h) {
   if (!h->have_forward) return fail(h, FDTD_ESTATE, "backward needs a preceding forward");
   if (layout_of(h, &h->fwd_rec).total > h->ws_bytes)
     return fail(h, FDTD_ENOMEM, "workspace too small for this record config");
-  int rc = begin(h);
+  return FDTD_OK;
+}
+
+static int backward_async(fdtd_handle* h, double seed, double seed2) {
+  int rc = backward_check(h);
+  if (rc) return rc;
+  rc = begin(h);
   if (rc) return rc;
   CK(h, upload_seeds(h, layout_of(h, &h->fwd_rec), seed, seed2, h->stream));
   int nl = 0;
@@ -2082,11 +2095,91 @@ extern "C" int fdtd_value_and_grad_host(fdtd_handle* h, const float* h_eps,
   return FDTD_OK;
 }
 
+// ------------------------------------------------------------ groups ----
+// The order in which the loops of a group start, and for each the loops whose end
+// it waits for.  A loop on a small grid leaves most of the GPU idle, so several run
+// side by side; but a grid's state is read again every half-step and comes from the
+// L2 cache only while it stays there, so loops run side by side only as long as
+// their states fit into kGroupCacheShare of it together (one that does not fit by
+// itself counts as most of it and leaves room to small ones).  The plan is a list
+// schedule over estimated times, longest state first, smaller loops filling the room
+// left.  Twenty cubes of 48^3 to 128^3, forward and backward: 107 ms all at once, 109
+// one after another, 94 so (98 with 1.3 of the cache).
+static const double kGroupCacheShare = 0.6;
+struct GroupSlot {
+  int i;                    // index in the call
+  std::vector<int> after;   // indices of the loops it waits for
+};
+static std::vector<GroupSlot> group_plan(fdtd_handle* const* hs, int n, int dir) {
+  int dev = 0, l2 = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess || l2 <= 0)
+    l2 = 128 << 20;
+  const double room = kGroupCacheShare * l2;
+  struct Loop { int i; double bytes, seconds; };
+  std::vector<Loop> todo;
+  for (int i = 0; i < n; ++i) {
+    const fdtd_handle* h = hs[i];
+    const double nc = (double)cells_of(h);
+    const double psi = 4.0 * (double)psi_layout(h, h->opt_compact && h->opt_kernel == 5).total;
+    const bool small = dir == 0 ? direct_forward(h) : direct_reverse(h);
+    // measured: microseconds a step and picoseconds a cell and step
+    const double step = dir == 0 ? (small ? 4.5e-6 + 8.5e-12 * nc : 15e-12 * nc)
+                                 : (small ? 6.5e-6 + 18.5e-12 * nc : 26e-12 * nc);
+    const double bytes = dir == 0 ? 28.0 * nc + psi : 52.0 * nc + 2.0 * psi;
+    todo.push_back({i, std::min(bytes, 0.8 * room), step * h->N});
+  }
+  std::stable_sort(todo.begin(), todo.end(),
+                   [](const Loop& a, const Loop& b) { return a.bytes > b.bytes; });
+  struct Run { double end, bytes; int i; };
+  std::vector<Run> running;
+  std::vector<GroupSlot> plan;
+  std::vector<int> freed;   // the loops whose end made the room there is now
+  double now = 0.0, used = 0.0;
+  while (!todo.empty()) {
+    for (size_t t = 0; t < todo.size();) {
+      if (used + todo[t].bytes > room && !running.empty()) {
+        ++t;
+        continue;
+      }
+      running.push_back({now + todo[t].seconds, todo[t].bytes, todo[t].i});
+      used += todo[t].bytes;
+      plan.push_back({todo[t].i, freed});
+      todo.erase(todo.begin() + t);
+    }
+    if (todo.empty()) break;
+    size_t e = 0;
+    for (size_t t = 1; t < running.size(); ++t)
+      if (running[t].end < running[e].end) e = t;
+    now = running[e].end;
+    used -= running[e].bytes;
+    // a later start also waits for what earlier ones of the same room waited for
+    freed.push_back(running[e].i);
+    if (freed.size() > 4) freed.erase(freed.begin());
+    running.erase(running.begin() + e);
+  }
+  return plan;
+}
+
+// Make the work queued next on h wait for the ends (event `end`) of the loops of a slot.
+static int group_wait(fdtd_handle* const* hs, const GroupSlot& s, int dir) {
+  fdtd_handle* h = hs[s.i];
+  int rc = ensure_cuda(h);
+  for (int j : s.after)
+    if (!rc) CK(h, cudaStreamWaitEvent(h->stream, dir == 0 ? hs[j]->t1 : hs[j]->t3, 0));
+  return rc;
+}
+
 extern "C" int fdtd_group_forward(fdtd_handle* const* hs, int n, const float* const* d_eps,
                                   const fdtd_record_cfg* rec, double* objs) {
   if (!hs || n < 0 || (n > 0 && (!d_eps || !objs))) return FDTD_EINVAL;
   for (int i = 0; i < n; ++i) {
-    int rc = forward_async(hs[i], d_eps[i], rec);
+    int rc = forward_check(hs[i], d_eps[i], rec);
+    if (rc) return rc;
+  }
+  for (const GroupSlot& s : group_plan(hs, n, 0)) {
+    int rc = group_wait(hs, s, 0);
+    if (!rc) rc = forward_async(hs[s.i], d_eps[s.i], rec);
     if (rc) return rc;
   }
   for (int i = 0; i < n; ++i) {
@@ -2101,7 +2194,12 @@ extern "C" int fdtd_group_backward(fdtd_handle* const* hs, int n, const double* 
   if (!hs || n < 0 || (n > 0 && (!seeds || !d_grads))) return FDTD_EINVAL;
   for (int i = 0; i < n; ++i) {
     if (!d_grads[i]) return fail(hs[i], FDTD_EINVAL, "gradient buffer is NULL");
-    int rc = backward_async(hs[i], seeds[i], 0.0);
+    int rc = backward_check(hs[i]);
+    if (rc) return rc;
+  }
+  for (const GroupSlot& s : group_plan(hs, n, 1)) {
+    int rc = group_wait(hs, s, 1);
+    if (!rc) rc = backward_async(hs[s.i], seeds[s.i], 0.0);
     if (rc) return rc;
   }
   for (int i = 0; i < n; ++i) {
