@@ -501,11 +501,12 @@ static bool two_step_forward(const fdtd_handle* h) {
 // Small grids run the direct half-steps (kernels_direct.cu) unless an option
 // names another form or shape.  The lines lie where they stop being faster
 // than the split staged ones (us per step, direct against split): forward 4.9 / 26.7
-// at 0.11 M cells, 14.5 / 30.5 at 1.2 M, 25.5 / 34.6 at 2.1 M, 38.2 / 43.8 at 2.9 M,
-// 50.6 / 50.5 at 3.4 M; reverse 6.7 / 30.6 at 0.11 M, 27.4 / 39.0 at 1.2 M, 51.8 / 56.7 at
-// 1.8 M, 64.6 / 60.4 at 2.1 M, 118 / 104 at 4 M (beyond the L2 cache its re-read
+// at 0.11 M cells, 14.5 / 30.5 at 1.2 M, 25.7 / 35.3 at 2.1 M, 41.5 / 47.2 at 3.2 M,
+// 55.1 / 60.9 at 4 M, 70.2 / 73.2 at 4.9 M, 77.1 / 80.8 at 5.8 M, 81.2 / 81.9 at 6 M, 99.0 /
+// 95.1 at 7.2 M; reverse 6.7 / 30.6 at 0.11 M, 27.2 / 39.0 at 1.2 M, 51.8 / 56.7 at
+// 1.8 M, 64.3 / 60.8 at 2.1 M, 118 / 104 at 4 M (beyond the L2 cache its re-read
 // neighbour planes come from HBM).
-static const long long kDirectForwardCells = 3400000, kDirectReverseCells = 2000000;
+static const long long kDirectForwardCells = 6000000, kDirectReverseCells = 2000000;
 static bool direct_shape(const fdtd_handle* h) {
   return h->opt_kernel == 5 && h->opt_tile_y == 8 && h->opt_tile_x == 32 && h->opt_stages == 2 &&
          h->opt_zchunk == 8 && h->opt_zchunk_fwd == -1 && h->opt_zgroups <= 1 && !h->opt_pdl &&

@@ -16,10 +16,17 @@
 //   * in the reverse phases the primal and the adjoint updates are separate
 //     blocks of one launch (twice the threads, half the registers).
 //
+// The forward's H half-step runs its planes up and its E half-step down, so
+// that each starts on the planes the other has just left in L2: on grids whose
+// state does not fit, part of every half-step still reads from L2 (us per step, both
+// up -> up and down: 60.3 -> 55.4 on 200 x 200 x 100, 76.5 -> 70.8 on 233 x 181 x 117,
+// 8.92 -> 8.84 on 100 x 100 x 50).  The reverse phases gain too little (118 -> 116 on
+// 200 x 200 x 100, where the staged ones take 104) and lose as much on small grids.
+//
 // Measured (GB300, us per forward / reverse step, split staged -> direct; the
 // CUDA graph's launches included): 48^3 with the FP32 tape of every step 26.7 /
-// 30.6 -> 5.2 / 6.9; 100 x 100 x 50 26.3 / 37.2 -> 10.0 / 15.7; 150 x 110 x 70 with
-// two detectors 30.6 / 39.0 -> 16.1 / 27.6, where it moves 93 (forward) and 188
+// 30.6 -> 4.9 / 6.7; 100 x 100 x 50 26.3 / 37.2 -> 8.8 / 14.9; 150 x 110 x 70 with
+// two detectors 30.6 / 39.0 -> 14.5 / 27.2, where it moves 93 (forward) and 188
 // (reverse) bytes per cell and step through L2, at 7 to 8 TB/s.
 //
 // Tape values in the half-steps: E^n of the high faces is recorded beside the
@@ -512,7 +519,7 @@ __global__ void __launch_bounds__(NT, 8) k_dir_fwd_e(const __grid_constant__ Dir
   float en[2][3], hh[2][3];
   const int zb = row - a.trows - a.drows;
   if (zb >= 0) {
-    const Pair p = pair_of(a, zb);
+    const Pair p = pair_of(a, a.g.nz - 1 - zb);   // down: see the head of this file
     if (!p.v0 || pair_on_det(a, p.x, p.y, p.z)) return;
     update_e<EX>(a, p.x, p.y, p.z, p.q, p.v1, en, hh);
     return;

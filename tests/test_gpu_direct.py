@@ -85,6 +85,23 @@ def test_direct_half_steps_equal_the_staged_ones(F, name, tape, k, interp, exact
     assert np.array_equal(a["grad"], b["grad"])
 
 
+@pytest.mark.parametrize("nx,ny,nz,direct", [(201, 173, 172, True), (202, 175, 171, False)])
+def test_the_largest_grids_of_the_direct_forward(F, nx, ny, nz, direct):
+    """Either side of the line (6 million cells): the same fields, tape and gradient as the
+    split half-steps, whichever form runs."""
+    from paper_2603_24027_gb300 import _capi as A
+    from paper_2603_24027_gb300 import inputs as I
+    w = I.ragged_box(nx=nx, ny=ny, nz=nz, P=9, n_steps=24)
+    rec = A.record_cfg("bf16", 3, "cubic")
+    a = _run(F, w, rec, {})
+    b = _run(F, w, rec, {A.OPT_FORWARD: 1, A.OPT_REVERSE: 1})
+    assert (a["launches"]["fwd_launches"] == 2 * w.n_steps) == direct
+    assert torch.equal(a["fields"], b["fields"])
+    skip, n = 128, 8 * w.n_steps * 2
+    assert np.array_equal(a["state"][skip:len(a["state"]) - n], b["state"][skip:len(b["state"]) - n])
+    assert np.array_equal(a["grad"], b["grad"])
+
+
 def test_sampled_timing_of_a_small_grid_keeps_its_kinds(F):
     """With kernel timing sampled, every kind has its own launch again; the results stay."""
     from paper_2603_24027_gb300 import _capi as A
