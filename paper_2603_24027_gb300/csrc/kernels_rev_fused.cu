@@ -117,6 +117,28 @@ constexpr int adj_ctas() { return MODE == 2 ? 4 : (MODE == 1 ? 5 : 6); }
 // tiles [ix0, ix1) x [iy0, iy1) and the chunks outside [iz0, iz1)
 // (zonly_chunk).  Ring units (MODE 2): a 1D grid over every chunk times the
 // ring tiles (ring_unit).
+//
+// Order of the primal and CPML-free launches (unit_order): groups of `rows` tile
+// rows, each with all its chunks before the next group.  A chunk reads two planes
+// of its z neighbours: on a wide grid, taken layer by layer over the whole plane,
+// the neighbour's were read 100 MB and more ago and come from HBM again.  rows is
+// chosen (group_rows) so that a layer of a group is about one wave of resident
+// CTAs: smaller groups run several layers side by side, which costs more than it
+// saves.  us per reverse step on 600 x 600 x 300, 19 x 75 tiles: 1957 (75 rows, one
+// group), 1937 (60), 1922 (44), 1924 (38), 1936 (30), 1967 (15); on 411 x 389 x 203 (13
+// x 49, the one group that the rule takes) 616, in groups of 38 rows 623, of 25 630.
+__device__ __forceinline__ int3 unit_order(int rows) {
+  const unsigned gx = gridDim.x, gz = gridDim.z, u = blockIdx.x + gx * (blockIdx.y + gridDim.y * blockIdx.z);
+  const unsigned per = gx * rows * gz, grp = u / per, r = u - grp * per;
+  const unsigned layer = gx * min((unsigned)rows, gridDim.y - grp * rows);   // the last group may be smaller
+  const unsigned z = r / layer, t = r - z * layer, y = t / gx;
+  return make_int3((int)(t - y * gx), (int)(grp * rows + y), (int)z);
+}
+inline int group_rows(dim3 grid) {
+  const unsigned wave = 750;   // five CTAs on each of 152 SMs
+  const unsigned n = (grid.x * grid.y + wave / 2) / wave;
+  return n > 1 ? (int)((grid.y + n - 1) / n) : (int)grid.y;
+}
 
 }  // namespace revf
 
@@ -128,12 +150,12 @@ using namespace revf;
 // that touch the interior's edge.
 template <int TY, int S, int TW, bool EX, bool FULL>
 __device__ __forceinline__ void rev_primal_unit(const RevMaps& m, const StepArgs& a,
-                                                unsigned char* dsm) {
+                                                unsigned char* dsm, int tix, int tiy, int cz) {
   typedef PL<TY, S, TW> Y;
   const Geo& g = a.g;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * (TW / 2) + tx;
-  const int x0 = (blockIdx.x + a.t0x) * TW, y0 = (blockIdx.y + a.t0y) * TY;
-  const int k0 = (blockIdx.z + a.zc0) * a.zchunk, k1 = min(g.nz, k0 + a.zchunk);
+  const int x0 = tix * TW, y0 = tiy * TY;
+  const int k0 = cz * a.zchunk, k1 = min(g.nz, k0 + a.zchunk);
   // task of this thread: the tile's pair (main), a pair of the +y halo row,
   // or a cell of the +x halo column (as the first cell of a pair)
   const bool mainT = ty < TY;
@@ -342,12 +364,13 @@ template <int TY, int S, int TW, bool EX>
 __global__ void __launch_bounds__(TW / 2 * (TY + 2), 6)
 k_rev_primal(const __grid_constant__ RevMaps m, const __grid_constant__ StepArgs a) {
   extern __shared__ __align__(128) unsigned char dsm[];
-  const int tix = blockIdx.x + a.t0x, tiy = blockIdx.y + a.t0y, cz = blockIdx.z + a.zc0;
+  const int3 u = unit_order(a.rows);
+  const int tix = u.x + a.t0x, tiy = u.y + a.t0y, cz = u.z + a.zc0;
   const RevUnits& U = a.U;
   if (tix >= U.ix0 && tix < U.ix1 && tiy >= U.iy0 && tiy < U.iy1 && cz >= U.iz0 && cz < U.iz1)
-    rev_primal_unit<TY, S, TW, EX, true>(m, a, dsm);
+    rev_primal_unit<TY, S, TW, EX, true>(m, a, dsm, tix, tiy, cz);
   else
-    rev_primal_unit<TY, S, TW, EX, false>(m, a, dsm);
+    rev_primal_unit<TY, S, TW, EX, false>(m, a, dsm, tix, tiy, cz);
 }
 
 // ============================================================= adjoint ===
@@ -364,10 +387,15 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, const __grid_constant__ StepArg
   int tix, tiy, cz;
   if (MODE == 2) {
     ring_unit(U, blockIdx.x, &tix, &tiy, &cz);
-  } else {
+  } else if (MODE == 1) {
     tix = blockIdx.x + a.t0x;
     tiy = blockIdx.y + a.t0y;
-    cz = MODE == 1 ? zonly_chunk(U, blockIdx.z) : blockIdx.z + a.zc0;
+    cz = zonly_chunk(U, blockIdx.z);
+  } else {
+    const int3 u = unit_order(a.rows);
+    tix = u.x + a.t0x;
+    tiy = u.y + a.t0y;
+    cz = u.z + a.zc0;
   }
   const int x0 = tix * TW, y0 = tiy * TY;
   const int k0 = cz * a.zchunk, k1 = min(g.nz, k0 + a.zchunk);
@@ -889,6 +917,7 @@ cudaError_t launch_rev_fused(int which, const RevMaps& m, const StepArgs& a, con
       return cudaErrorInvalidValue;
   }
   if (grid.x == 0 || grid.y == 0 || grid.z == 0) return cudaSuccess;
+  b.rows = group_rows(grid);
   return launch_rev_fused_t<8>(which, m, b, U, grid, s);
 }
 
