@@ -113,10 +113,11 @@ template <int S, int MODE>
 constexpr int adj_ctas() { return MODE == 2 ? 4 : (MODE == 1 ? 5 : 6); }
 
 // Tile and chunk of a unit.  Primal and CPML-free adjoint launches: a 3D
-// grid offset by (t0x, t0y, zc0).  z-only units (MODE 1): a 3D grid over the
+// grid offset by (t0x, t0y).  z-only units (MODE 1): a 3D grid over the
 // tiles [ix0, ix1) x [iy0, iy1) and the chunks outside [iz0, iz1)
 // (zonly_chunk).  Ring units (MODE 2): a 1D grid over every chunk times the
-// ring tiles (ring_unit).
+// ring tiles (ring_unit).  A launch covers the planes [zb, ze) in chunks of zl
+// (launch_chunk).
 //
 // Order of the primal and CPML-free launches (unit_order): groups of `rows` tile
 // rows, each with all its chunks before the next group.  A chunk reads two planes
@@ -139,6 +140,18 @@ inline int group_rows(dim3 grid) {
   const unsigned n = (grid.x * grid.y + wave / 2) / wave;
   return n > 1 ? (int)((grid.y + n - 1) / n) : (int)grid.y;
 }
+// Planes per chunk of a launch; zc: the chunk that the units are counted in.  Every
+// chunk streams two planes more than it owns, and a ring unit streams its
+// auxiliaries' and profiles' too: three times zc there (us per reverse step, ring
+// chunks of 8 / 24 / 32 / 64 planes: 1929 / 1893 / 1889 / 1884 on 600 x 600 x 300, 617 /
+// 609 / 608 / 611 on 411 x 389 x 203, 200 / 194 / 194 / 203 on 301 x 203 x 151, 151 /
+// 149 / 152 / - on 200 x 200 x 150, where one CTA's chain of planes begins to show).
+// The primal units take twice zc where they run in groups of tile rows (1887 -> 1878 on
+// 600 x 600 x 300, 893 -> 886 on 800 x 700 x 90; one group: no difference).  The
+// CPML-free adjoint units gain nothing (16 planes: 1927 against 1929; 24: 1967).
+inline int launch_chunk(int which, int zc, bool groups) {
+  return which == 3 ? 3 * zc : (which == 0 && groups ? 2 * zc : zc);
+}
 
 }  // namespace revf
 
@@ -155,7 +168,7 @@ __device__ __forceinline__ void rev_primal_unit(const RevMaps& m, const StepArgs
   const Geo& g = a.g;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * (TW / 2) + tx;
   const int x0 = tix * TW, y0 = tiy * TY;
-  const int k0 = cz * a.zchunk, k1 = min(g.nz, k0 + a.zchunk);
+  const int k0 = a.zb + cz * a.zl, k1 = min(a.ze, k0 + a.zl);
   // task of this thread: the tile's pair (main), a pair of the +y halo row,
   // or a cell of the +x halo column (as the first cell of a pair)
   const bool mainT = ty < TY;
@@ -365,12 +378,12 @@ __global__ void __launch_bounds__(TW / 2 * (TY + 2), 6)
 k_rev_primal(const __grid_constant__ RevMaps m, const __grid_constant__ StepArgs a) {
   extern __shared__ __align__(128) unsigned char dsm[];
   const int3 u = unit_order(a.rows);
-  const int tix = u.x + a.t0x, tiy = u.y + a.t0y, cz = u.z + a.zc0;
+  const int tix = u.x + a.t0x, tiy = u.y + a.t0y, k0 = a.zb + u.z * a.zl;
   const RevUnits& U = a.U;
-  if (tix >= U.ix0 && tix < U.ix1 && tiy >= U.iy0 && tiy < U.iy1 && cz >= U.iz0 && cz < U.iz1)
-    rev_primal_unit<TY, S, TW, EX, true>(m, a, dsm, tix, tiy, cz);
+  if (tix >= U.ix0 && tix < U.ix1 && tiy >= U.iy0 && tiy < U.iy1 && k0 >= a.zi0 && min(a.ze, k0 + a.zl) <= a.zi1)
+    rev_primal_unit<TY, S, TW, EX, true>(m, a, dsm, tix, tiy, u.z);
   else
-    rev_primal_unit<TY, S, TW, EX, false>(m, a, dsm, tix, tiy, cz);
+    rev_primal_unit<TY, S, TW, EX, false>(m, a, dsm, tix, tiy, u.z);
 }
 
 // ============================================================= adjoint ===
@@ -395,10 +408,10 @@ k_rev_adjoint(const __grid_constant__ RevMaps m, const __grid_constant__ StepArg
     const int3 u = unit_order(a.rows);
     tix = u.x + a.t0x;
     tiy = u.y + a.t0y;
-    cz = u.z + a.zc0;
+    cz = u.z;
   }
   const int x0 = tix * TW, y0 = tiy * TY;
-  const int k0 = cz * a.zchunk, k1 = min(g.nz, k0 + a.zchunk);
+  const int k0 = a.zb + cz * a.zl, k1 = min(a.ze, k0 + a.zl);
   // task: the tile's pair (main), a pair of the -y halo row, or a cell of the
   // -x halo column (as the second cell of a pair)
   const bool mainT = ty < TY;
@@ -896,28 +909,41 @@ cudaError_t launch_rev_fused(int which, const RevMaps& m, const StepArgs& a, con
   dim3 grid(0, 0, 0);
   StepArgs b = a;
   b.U = U;
-  const int nzin = U.iz1 - U.iz0;
+  const int nzin = U.iz1 - U.iz0, zc = a.zchunk, nz = a.g.nz;
+  b.zi0 = U.iz0 * zc;
+  b.zi1 = min(nz, U.iz1 * zc);
+  auto chunks = [&](int z0, int z1, int zl) {
+    b.zb = z0;
+    b.ze = z1;
+    b.zl = zl;
+    return z1 > z0 ? (unsigned)((z1 - z0 + zl - 1) / zl) : 0u;
+  };
   switch (which) {
     case 0:
-      grid = dim3(U.px1 - U.px0, U.py1 - U.py0, U.pz1 - U.pz0);
-      b.t0x = U.px0; b.t0y = U.py0; b.zc0 = U.pz0;
+      grid = dim3(U.px1 - U.px0, U.py1 - U.py0, 1);
+      b.rows = group_rows(grid);
+      grid.z = chunks(U.pz0 * zc, min(nz, U.pz1 * zc),
+                      launch_chunk(0, zc, b.rows < (int)grid.y));
+      b.t0x = U.px0; b.t0y = U.py0;
       break;
     case 1:
-      grid = dim3(U.ix1 - U.ix0, U.iy1 - U.iy0, nzin);
-      b.t0x = U.ix0; b.t0y = U.iy0; b.zc0 = U.iz0;
+      grid = dim3(U.ix1 - U.ix0, U.iy1 - U.iy0, 1);
+      b.rows = group_rows(grid);
+      grid.z = chunks(b.zi0, b.zi1, launch_chunk(1, zc, false));
+      b.t0x = U.ix0; b.t0y = U.iy0;
       break;
     case 2:
+      chunks(0, nz, zc);
       grid = dim3(U.ix1 - U.ix0, U.iy1 - U.iy0, U.nzc - nzin);
-      b.t0x = U.ix0; b.t0y = U.iy0; b.zc0 = 0;
+      b.t0x = U.ix0; b.t0y = U.iy0;
       break;
     case 3:
-      grid = dim3((unsigned)(ring_tiles(U) * U.nzc), 1, 1);
+      grid = dim3((unsigned)(ring_tiles(U) * chunks(0, nz, launch_chunk(3, zc, false))), 1, 1);
       break;
     default:
       return cudaErrorInvalidValue;
   }
   if (grid.x == 0 || grid.y == 0 || grid.z == 0) return cudaSuccess;
-  b.rows = group_rows(grid);
   return launch_rev_fused_t<8>(which, m, b, U, grid, s);
 }
 
