@@ -43,6 +43,8 @@ struct DirectArgs {
   const float* scales;
   Interp ip;
   unsigned* err;
+  int dep;             // launch as a programmatic dependent (0: sampled timing, which needs
+                       // each launch's own time)
   // set by launch_direct
   DirectBox sbox, dbox, dbox2;   // source and detector planes
   int trows, drows;              // grid rows of tape blocks, of detector blocks (forward E)

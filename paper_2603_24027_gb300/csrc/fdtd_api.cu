@@ -84,6 +84,7 @@ struct fdtd_handle {
   char* ws;
   size_t ws_bytes;
   bool tables_uploaded;
+  bool one_stream;            // the no-allocation call: every launch on the caller's stream
   bool have_forward;
   int fwd_buf;                // field buffer holding the state after forward
   fdtd_record_cfg fwd_rec;
@@ -509,7 +510,7 @@ static bool two_step_forward(const fdtd_handle* h) {
 static const long long kDirectForwardCells = 6000000, kDirectReverseCells = 2000000;
 static bool direct_shape(const fdtd_handle* h) {
   return h->opt_kernel == 5 && h->opt_tile_y == 8 && h->opt_tile_x == 32 && h->opt_stages == 2 &&
-         h->opt_zchunk == 8 && h->opt_zchunk_fwd == -1 && h->opt_zgroups <= 1 && !h->opt_pdl &&
+         h->opt_zchunk == 8 && h->opt_zchunk_fwd == -1 && h->opt_zgroups == 0 && !h->opt_pdl &&
          !h->opt_prefetch;
 }
 static Geo geo_of(const fdtd_handle* h);
@@ -769,6 +770,7 @@ extern "C" int fdtd_create(const fdtd_grid* grid, double dx, double dt, const fd
   h->opt_zchunk_fwd = -1;
   h->opt_zchunk_fwd2 = -1;
   h->opt_zgroups = 0;
+  h->one_stream = false;
   h->zfork = nullptr;
   h->opt_sample = 0;
   h->opt_stages = 2;
@@ -1056,6 +1058,7 @@ static Det det2_of(const fdtd_handle* h) { return det_of(h->det2); }
 // step's restore, so only two phases overlap there).
 static int zgroups_of(const fdtd_handle* h, int dir) {
   if (h->opt_kernel != 5) return 1;
+  if (h->one_stream) return 1;
   if (h->opt_zgroups > 0) return h->opt_zgroups;
   return dir == 0 ? 4 : 3;
 }
@@ -1127,6 +1130,7 @@ static DirectArgs direct_args(const fdtd_handle* h, const Layout& L, const StepA
   d.xq = a.xq; d.xs = a.xs; d.xi = a.xi;
   d.fc = h->faces;
   d.err = a.err;
+  d.dep = h->opt_sample == 0;
   return d;
 }
 
@@ -1439,8 +1443,8 @@ static cudaError_t enqueue_forward(fdtd_handle* h, const fdtd_record_cfg* rec, i
     // 300, us per forward step with 4, 8 and 16 chunks: 1055, 1036, 1028, with the
     // split half-steps outside the deep box)
     const int zdeep = h->opt_zchunk_fwd2 > 0 ? h->opt_zchunk_fwd2 : 16 * zcs;
-    const bool conc = h->opt_sample == 0 && h->opt_zgroups != 1 && h->zs.size() >= 3 &&
-                      h->zev.size() >= 9;
+    const bool conc = h->opt_sample == 0 && h->opt_zgroups != 1 && !h->one_stream &&
+                      h->zs.size() >= 3 && h->zev.size() >= 9;
     int cur = lent ? (h->N & 1) : 0, ps = 0;
     if (cur == 1 && (e = cudaMemsetAsync(h->ws + fo[1], 0, nc6, h->stream))) return e;
     // The launches of step n from buffer i into buffer o over the kinds [first, 5)
@@ -1631,8 +1635,8 @@ static cudaError_t enqueue_backward(fdtd_handle* h, const fdtd_record_cfg* rec, 
   const RevUnits U = rev_units(a.g, a.zchunk);
   // the adjoint launches run on a side stream unless kernel timing is being
   // sampled or one launch per half-step is asked for (FDTD_OPT_ZGROUPS = 1)
-  const bool conc = fused && h->opt_sample == 0 && h->opt_zgroups != 1 && h->zs.size() >= 3 &&
-                    h->zev.size() >= 9;
+  const bool conc = fused && h->opt_sample == 0 && h->opt_zgroups != 1 && !h->one_stream &&
+                    h->zs.size() >= 3 && h->zev.size() >= 9;
   for (int b = 0; fused && b < 2; ++b)
     if ((e = encode_rev_maps((const float*)(h->ws + L.F[b]), (const float*)(h->ws + L.L[b]),
                              (const float*)(h->ws + L.cb), (const float*)(h->ws + L.psiL[b]), a.g,
@@ -2910,12 +2914,12 @@ extern "C" int fdtd_value_and_grad_noalloc(fdtd_handle* h, const float* d_eps,
   size_t b0 = h->ws_bytes;
   bool up0 = h->tables_uploaded;
   cudaStream_t s0 = h->stream;
-  int samp0 = h->opt_sample, zg0 = h->opt_zgroups;   // no side streams here
+  int samp0 = h->opt_sample;
   h->ws = (char*)scratch;
   h->ws_bytes = FDTD_NOALLOC_SCRATCH_BYTES;
   h->stream = h->user_stream;
   h->opt_sample = 0;
-  h->opt_zgroups = 1;
+  h->one_stream = true;
   h->have_forward = false;
   auto restore = [&]() {
     h->ws = ws0;
@@ -2923,7 +2927,7 @@ extern "C" int fdtd_value_and_grad_noalloc(fdtd_handle* h, const float* d_eps,
     h->tables_uploaded = up0;
     h->stream = s0;
     h->opt_sample = samp0;
-    h->opt_zgroups = zg0;
+    h->one_stream = false;
     h->have_forward = false;
   };
   auto run = [&]() -> int {

@@ -1031,7 +1031,7 @@ static cudaError_t launch_dep(KT kernel, dim3 grid, cudaStream_t s, const Direct
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = a.dep ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
