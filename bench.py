@@ -460,6 +460,10 @@ def run_ours(args):
     total_wall = max_over_ranks(sum(wall_s), ws, dev)
     t = sim.last_timing()
     gpu_launches = (t["fwd_launches"] + t["bwd_launches"] + 2) * args.steps
+    # small grids: two launches per forward step (the sampled pass below, one z group by
+    # name, runs and times the split half-steps)
+    direct_forward = (args.zgroups == 0 and args.forward < 1 and
+                      t["fwd_launches"] <= 2 * w.n_steps + w.n_steps // rec.k + 1)
     cell_updates = w.n_cells * w.n_steps
     value = job_rate(ws, cell_updates, args.steps, total_ms / 1e3)
 
@@ -515,7 +519,8 @@ def run_ours(args):
                    "parallelism": f"replicas x{ws}",
                    "l2": "state larger than L2; L2 also flushed before every timed step",
                    "zgroups": args.zgroups or "automatic",
-                   "forward_step": ("two steps per pass over the deep units" if "fwd_2step" in kern
+                   "forward_step": ("direct" if direct_forward else
+                                    "two steps per pass over the deep units" if "fwd_2step" in kern
                                     else "fused" if "fwd_fused" in kern else "split"),
                    "reverse_step": "fused" if "rev_primal" in kern else "split",
                    "autotuned": None if tuned is None else

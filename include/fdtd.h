@@ -193,8 +193,9 @@ int fdtd_value_and_grad_host(fdtd_handle* h, const float* h_eps, const fdtd_reco
 /* Batched designs: n independent handles (each with its own workspace)
  * processed together; objs[i] / d_grads[i] as in fdtd_forward/backward.
  * Each handle runs its own time loop (a CUDA graph on its own stream); all
- * are enqueued before any is awaited.  They run concurrently as far as their
- * states share the L2 cache; the others wait on the device for room. */
+ * are enqueued before any is awaited.  The forwards run concurrently as far as
+ * their states share the L2 cache, the others waiting on the device for room;
+ * the backwards all run concurrently. */
 int fdtd_group_forward(fdtd_handle* const* hs, int n, const float* const* d_eps,
                        const fdtd_record_cfg* rec, double* objs);
 int fdtd_group_backward(fdtd_handle* const* hs, int n, const double* seeds,

@@ -42,7 +42,7 @@ struct Layout {
 struct GraphKey {
   int dir, dtype, k, interp, scaled, kernel, tile_y, zchunk, sample, stages, pdl, prefetch,
       tile_x, compact, exact, coeffs, zchunk_fwd, zgroups, inject_wait, reverse, forward,
-      zchunk_fwd2, start_buf;
+      zchunk_fwd2, start_buf, group_split;
   bool operator<(const GraphKey& o) const {
     return memcmp(this, &o, sizeof(GraphKey)) < 0;
   }
@@ -84,6 +84,7 @@ struct fdtd_handle {
   char* ws;
   size_t ws_bytes;
   bool tables_uploaded;
+  bool group_split;           // this loop of a group call takes the split reverse phases
   bool one_stream;            // the no-allocation call: every launch on the caller's stream
   bool have_forward;
   int fwd_buf;                // field buffer holding the state after forward
@@ -519,7 +520,7 @@ static bool direct_forward(const fdtd_handle* h) {
          (long long)h->nx * h->ny * h->nz <= kDirectForwardCells;
 }
 static bool direct_reverse(const fdtd_handle* h) {
-  return direct_shape(h) && direct_fits(geo_of(h)) && h->opt_reverse == 0 &&
+  return !h->group_split && direct_shape(h) && direct_fits(geo_of(h)) && h->opt_reverse == 0 &&
          (long long)h->nx * h->ny * h->nz <= kDirectReverseCells;
 }
 
@@ -532,8 +533,8 @@ static bool direct_reverse(const fdtd_handle* h) {
 // per step, forward split / fused / two steps: 60 / 73 / 85 on 200 x 200 x 100 (4 M
 // cells), 127 / 132 / 141 on 301 x 203 x 151 (9.2 M), 144 / 147 / 133 on 300 x 300 x
 // 120 (10.8 M), 176 / 175 / 153 on 300 x 300 x 150 (13.5 M), 406 / - / 315 on 411 x
-// 389 x 203 (32 M); reverse split / fused: 95 / 89 on 180 x 180 x 100, 158 / 150 on
-// 200 x 200 x 150, 224 / 200 (9.2 M), 319 / 287 (13.5 M), 717 / 611 (32 M).  An
+// 389 x 203 (32 M); reverse split / fused: 159 / 149 on 200 x 200 x 150 (6 M),
+// 196 / 178 on 260 x 200 x 150, 224 / 194 (9.2 M), 717 / 602 (32 M).  An
 // option that names another shape of the split half-steps leaves the choice to the
 // units' CPML share alone.
 enum ForwardForm { kSplit, kDirect, kFusedStep, kTwoStep };
@@ -771,6 +772,7 @@ extern "C" int fdtd_create(const fdtd_grid* grid, double dx, double dt, const fd
   h->opt_zchunk_fwd2 = -1;
   h->opt_zgroups = 0;
   h->one_stream = false;
+  h->group_split = false;
   h->zfork = nullptr;
   h->opt_sample = 0;
   h->opt_stages = 2;
@@ -1831,6 +1833,7 @@ static int run_loop(fdtd_handle* h, const fdtd_record_cfg* rec, int dir, Enqueue
   key.reverse = h->opt_reverse;
   key.forward = h->opt_forward;
   key.zchunk_fwd2 = h->opt_zchunk_fwd2;
+  key.group_split = dir == 1 && h->group_split;
   key.start_buf = dir == 1 ? h->fwd_buf : 0;   // the backward starts from the forward's buffer
   auto it = h->graphs.find(key);
   if (it == h->graphs.end()) {
@@ -2101,21 +2104,22 @@ extern "C" int fdtd_value_and_grad_host(fdtd_handle* h, const float* h_eps,
 }
 
 // ------------------------------------------------------------ groups ----
-// The order in which the loops of a group start, and for each the loops whose end
-// it waits for.  A loop on a small grid leaves most of the GPU idle, so several run
+// The order in which the loops of a group's forward start, and for each the loops
+// whose end it waits for.  A loop on a small grid leaves most of the GPU idle, so several run
 // side by side; but a grid's state is read again every half-step and comes from the
 // L2 cache only while it stays there, so loops run side by side only as long as
 // their states fit into kGroupCacheShare of it together (one that does not fit by
 // itself counts as most of it and leaves room to small ones).  The plan is a list
 // schedule over estimated times, longest state first, smaller loops filling the room
-// left.  Twenty cubes of 48^3 to 128^3, forward and backward: 107 ms all at once, 109
-// one after another, 94 so (98 with 1.3 of the cache).
+// left.  ms for twenty cubes of 48^3 to 128^3 / sixty-four of 32^3 to 128^3: 30.5 / 732
+// with 0.6 of the cache, 33.5 / 735 with 0.3, 31.6 / 691 with 1.0, 35.1 / 784 with 2, 35.5
+// / 811 all at once.
 static const double kGroupCacheShare = 0.6;
 struct GroupSlot {
   int i;                    // index in the call
   std::vector<int> after;   // indices of the loops it waits for
 };
-static std::vector<GroupSlot> group_plan(fdtd_handle* const* hs, int n, int dir) {
+static std::vector<GroupSlot> group_plan(fdtd_handle* const* hs, int n) {
   int dev = 0, l2 = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess || l2 <= 0)
@@ -2127,11 +2131,9 @@ static std::vector<GroupSlot> group_plan(fdtd_handle* const* hs, int n, int dir)
     const fdtd_handle* h = hs[i];
     const double nc = (double)cells_of(h);
     const double psi = 4.0 * (double)psi_layout(h, h->opt_compact && h->opt_kernel == 5).total;
-    const bool small = dir == 0 ? direct_forward(h) : direct_reverse(h);
-    // measured: microseconds a step and picoseconds a cell and step
-    const double step = dir == 0 ? (small ? 4.5e-6 + 8.5e-12 * nc : 15e-12 * nc)
-                                 : (small ? 6.5e-6 + 18.5e-12 * nc : 26e-12 * nc);
-    const double bytes = dir == 0 ? 28.0 * nc + psi : 52.0 * nc + 2.0 * psi;
+    // measured: seconds a step and a cell and step
+    const double step = direct_forward(h) ? 4.5e-6 + 8.5e-12 * nc : 15e-12 * nc;
+    const double bytes = 28.0 * nc + psi;
     todo.push_back({i, std::min(bytes, 0.8 * room), step * h->N});
   }
   std::stable_sort(todo.begin(), todo.end(),
@@ -2166,12 +2168,12 @@ static std::vector<GroupSlot> group_plan(fdtd_handle* const* hs, int n, int dir)
   return plan;
 }
 
-// Make the work queued next on h wait for the ends (event `end`) of the loops of a slot.
-static int group_wait(fdtd_handle* const* hs, const GroupSlot& s, int dir) {
+// Make the work queued next on h wait for the ends of the loops of a slot.
+static int group_wait(fdtd_handle* const* hs, const GroupSlot& s) {
   fdtd_handle* h = hs[s.i];
   int rc = ensure_cuda(h);
   for (int j : s.after)
-    if (!rc) CK(h, cudaStreamWaitEvent(h->stream, dir == 0 ? hs[j]->t1 : hs[j]->t3, 0));
+    if (!rc) CK(h, cudaStreamWaitEvent(h->stream, hs[j]->t1, 0));
   return rc;
 }
 
@@ -2182,8 +2184,8 @@ extern "C" int fdtd_group_forward(fdtd_handle* const* hs, int n, const float* co
     int rc = forward_check(hs[i], d_eps[i], rec);
     if (rc) return rc;
   }
-  for (const GroupSlot& s : group_plan(hs, n, 0)) {
-    int rc = group_wait(hs, s, 0);
+  for (const GroupSlot& s : group_plan(hs, n)) {
+    int rc = group_wait(hs, s);
     if (!rc) rc = forward_async(hs[s.i], d_eps[s.i], rec);
     if (rc) return rc;
   }
@@ -2194,6 +2196,15 @@ extern "C" int fdtd_group_forward(fdtd_handle* const* hs, int n, const float* co
   return FDTD_OK;
 }
 
+// The loops of a group's backward all start at once, the largest first.  When the
+// group has more cells than a single direct reverse takes, those of grids above the
+// size below run as split phases: side by side they fill the GPU anyway, and what
+// counts then is the bytes read through L2, where the staged phases read less.  ms
+// for twenty cubes of 48^3 to 128^3 / sixty-four of 32^3 to 128^3: 59 / 1366; the split
+// phases on every grid 62 / 1428; the direct ones by size alone 71 / 1456, and with the
+// forward's plan 65 / 1532; in the order of the call 62 / 1371.
+static const long long kGroupDirectReverseCells = 200000;
+
 extern "C" int fdtd_group_backward(fdtd_handle* const* hs, int n, const double* seeds,
                                    float* const* d_grads) {
   if (!hs || n < 0 || (n > 0 && (!seeds || !d_grads))) return FDTD_EINVAL;
@@ -2202,9 +2213,18 @@ extern "C" int fdtd_group_backward(fdtd_handle* const* hs, int n, const double* 
     int rc = backward_check(hs[i]);
     if (rc) return rc;
   }
-  for (const GroupSlot& s : group_plan(hs, n, 1)) {
-    int rc = group_wait(hs, s, 1);
-    if (!rc) rc = backward_async(hs[s.i], seeds[s.i], 0.0);
+  long long cells = 0;
+  std::vector<int> order(n);
+  for (int i = 0; i < n; ++i) {
+    cells += cells_of(hs[i]);
+    order[i] = i;
+  }
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int a, int b) { return cells_of(hs[a]) > cells_of(hs[b]); });
+  for (int i : order) {
+    hs[i]->group_split = cells > kDirectReverseCells && cells_of(hs[i]) > kGroupDirectReverseCells;
+    int rc = backward_async(hs[i], seeds[i], 0.0);
+    hs[i]->group_split = false;
     if (rc) return rc;
   }
   for (int i = 0; i < n; ++i) {

@@ -35,14 +35,16 @@
 // operations exactly, so the primal fields are bit-identical to the split
 // kernels', and so are the adjoint's (explicitly rounded products and sums).
 //
-// What bounds them: DRAM for the launches together (600 x 600 x 300: 12.2 GB per
-// reverse step in 1974 us, 6.2 TB/s, 0.91 of the measured copy), and before
+// What bounds them: DRAM for the launches together (600 x 600 x 300: 11.7 GB per
+// reverse step in 1879 us, 6.24 TB/s, 0.92 of the measured copy), and before
 // that the instructions per cell.  The primal units inside the interior carry no
 // predicate (FULL), the exchange between the two half-steps happens in the
 // staged box itself, one block barrier per plane is left in the primal and two
 // in the adjoint (three before), and stores address a plane's uniform base with a
 // 32-bit offset: 2071 -> 1974 us per reverse step (600 x 600 x 300), 671 -> 639
-// (411 x 389 x 203), 239 -> 218 (301 x 203 x 151).
+// (411 x 389 x 203), 239 -> 218 (301 x 203 x 151).  A stream for each launch (in
+// fdtd_api.cu), the order of the units and the chunks' lengths (group_rows,
+// launch_chunk) took it to 1879, 602 and 194.
 #include <cudaTypedefs.h>
 
 #include "lag_common.cuh"
