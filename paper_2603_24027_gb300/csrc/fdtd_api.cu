@@ -59,6 +59,7 @@ struct SampleEntry {
 struct GraphEntry {
   cudaGraphExec_t exec;
   std::vector<SampleEntry> plan;   // intervals the graph's event nodes record
+  int launches;                    // its kernel launches
 };
 
 struct BatchPlan;
@@ -1849,14 +1850,13 @@ static int run_loop(fdtd_handle* h, const fdtd_record_cfg* rec, int dir, Enqueue
     cudaGraphDestroy(graph);
     if (e3) return cuda_fail(h, "cudaGraphInstantiate", e3);
     if (h->graphs.size() >= 8) drop_graphs(h);
-    it = h->graphs.insert(std::make_pair(key, GraphEntry{exec, h->splan[dir]})).first;
-    if (dir == 0) h->launches_fwd = nl; else h->launches_bwd = nl;
+    it = h->graphs.insert(std::make_pair(key, GraphEntry{exec, h->splan[dir], nl})).first;
   }
   h->splan[dir] = it->second.plan;
   CK(h, cudaEventRecord(ta, h->stream));
   CK(h, cudaGraphLaunch(it->second.exec, h->stream));
   CK(h, cudaEventRecord(tb, h->stream));
-  *launches = dir == 0 ? h->launches_fwd : h->launches_bwd;
+  *launches = it->second.launches;
   return FDTD_OK;
 }
 

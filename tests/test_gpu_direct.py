@@ -102,6 +102,32 @@ def test_the_largest_grids_of_the_direct_forward(F, nx, ny, nz, direct):
     assert np.array_equal(a["grad"], b["grad"])
 
 
+@pytest.mark.parametrize("sizes,split", [((44, 60, 128), {60, 128}),   # above 2 million cells
+                                         ((44, 60, 96), set())])       # below
+def test_a_groups_backward_equals_each_handles_own(F, sizes, split):
+    """A large group's backward runs its larger grids as split phases; the gradients stay the
+    own runs', whose form a group call does not change."""
+    from paper_2603_24027_gb300 import _capi as A
+    from paper_2603_24027_gb300 import inputs as I
+    ws = [I.ragged_box(nx=n, ny=n, nz=n, P=7, n_steps=31, seed=n) for n in sizes]
+    rec = A.record_cfg("bf16", 3)
+    eps = [torch.from_numpy(w.eps).cuda() for w in ws]
+    sims = [F.Simulation(w, device="cuda") for w in ws]
+    own = []
+    for s, e in zip(sims, eps):
+        s.forward(e, rec)
+        own.append((s.backward(0.5).clone(), s.last_timing()["bwd_launches"]))
+    F.group_forward(sims, eps, rec)
+    grads = F.group_backward(sims, [0.5] * len(sims))
+    for w, s, g, (g0, n0) in zip(ws, sims, grads, own):
+        assert torch.equal(g, g0)
+        assert (s.last_timing()["bwd_launches"] > 2 * w.n_steps + 1) == (w.nx in split)
+    for s, e, (g0, n0) in zip(sims, eps, own):
+        s.forward(e, rec)
+        assert torch.equal(s.backward(0.5), g0)
+        assert s.last_timing()["bwd_launches"] == n0
+
+
 def test_sampled_timing_of_a_small_grid_keeps_its_kinds(F):
     """With kernel timing sampled, every kind has its own launch again; the results stay."""
     from paper_2603_24027_gb300 import _capi as A
