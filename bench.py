@@ -230,6 +230,10 @@ PHASE_KERNELS = {"forward": ["fwd_fused", "fwd_2step", "fwd_h", "fwd_e", "record
                              "rev_adjoint_cpml"]}
 
 
+STEP_LABELS = {"direct": "direct", "split": "split", "fused": "fused",
+               "two_step": "two steps per pass over the deep units"}
+
+
 def read_peaks():
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     try:
@@ -358,34 +362,62 @@ def apply_options(A, sim, args):
         sim.set_option(A.OPT_USE_GRAPHS, 0)
 
 
-def sampled_breakdown(A, fdtd, args, w, rec, dev, flush):
-    """Per-kernel in-loop costs from a pass with one launch per half-step on
-    the workload shortened to --sample-steps time steps (same grid, same work
-    per launch): CUDA events on the library's stream around sampled launches
-    (pair-minus-single intervals, see fdtd_kernel_timing)."""
+def sampled_passes(A, forms):
+    """The sampled runs that time the kernels of the step forms `forms` (those of the
+    timed run): [(directions, extra options)].  Sampling records split half-steps only
+    with one launch each (one z group), and that option would take a grid off the
+    other automatic forms; so each direction that runs split is named as split and run
+    with one z group, and the others keep the timed run's options."""
+    split = {"forward": A.OPT_FORWARD, "reverse": A.OPT_REVERSE}
+    as_split = [d for d in split if forms[d] == "split"]
+    as_timed = [d for d in split if forms[d] != "split"]
+    passes = []
+    if as_timed:
+        passes.append((as_timed, {}))
+    if as_split:
+        passes.append((as_split, {A.OPT_ZGROUPS: 1, **{split[d]: 1 for d in as_split}}))
+    return passes
+
+
+def sampled_breakdown(A, fdtd, args, w, rec, dev, flush, sim_options):
+    """Per-kernel in-loop costs on the workload shortened to --sample-steps
+    time steps (same grid, same work per launch, same step forms): CUDA
+    events on the library's stream around sampled launches (pair-minus-single
+    intervals, see fdtd_kernel_timing)."""
     import torch
     ws_ = w.replace(n_steps=max(1, min(w.n_steps, args.sample_steps)))
-    sim = fdtd.Simulation(ws_, device=dev)
-    apply_options(A, sim, args)
-    sim.set_option(A.OPT_ZGROUPS, 1)
-    sim.set_option(A.OPT_SAMPLE_EVERY, args.sample_every)
     eps = torch.from_numpy(ws_.eps).to(dev)
-    sim.forward(eps, rec)                   # capture the sampled graphs
-    sim.backward(1.0)
-    torch.cuda.synchronize()
-    ktimes, loop_ms = {}, []
-    for _ in range(2):
-        flush.random_(0, 255)
-        sim.forward(eps, rec)
+    ktimes, loop_ms = {}, {"forward": [], "reverse": []}
+    probe = fdtd.Simulation(ws_, device=dev)
+    sim_options(probe)
+    forms = probe.step_forms()
+    del probe
+    for directions, options in sampled_passes(A, forms):
+        sim = fdtd.Simulation(ws_, device=dev)
+        sim_options(sim)
+        for opt, val in options.items():
+            sim.set_option(opt, val)
+        sim.set_option(A.OPT_SAMPLE_EVERY, args.sample_every)
+        assert all(sim.step_forms()[d] == forms[d] for d in directions)
+        sim.forward(eps, rec)                   # capture the sampled graphs
         sim.backward(1.0)
-        t = sim.last_timing()
-        loop_ms.append(t["fwd_ms"] + t["bwd_ms"])
-        for name, (ms, n) in sim.kernel_timing().items():
-            ktimes.setdefault(name, []).append((ms, n))
-    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        for _ in range(2):
+            flush.random_(0, 255)
+            sim.forward(eps, rec)
+            sim.backward(1.0)
+            t = sim.last_timing()
+            for d, key in (("forward", "fwd_ms"), ("reverse", "bwd_ms")):
+                if d in directions:
+                    loop_ms[d].append(t[key])
+            for name, (ms, n) in sim.kernel_timing().items():
+                if any(name in PHASE_KERNELS[d] for d in directions):
+                    ktimes.setdefault(name, []).append((ms, n))
+        torch.cuda.synchronize()
+        del sim
     per_step = {"record": 1.0 / rec.k, "fwd_2step": 0.5}
     kb = kernel_bytes(w)
-    step_ms = statistics.median(loop_ms) / ws_.n_steps
+    step_ms = sum(statistics.median(v) for v in loop_ms.values()) / ws_.n_steps
     kern = {}
     for name, lst in ktimes.items():
         n = sum(c for _, c in lst)
@@ -400,8 +432,7 @@ def sampled_breakdown(A, fdtd, args, w, rec, dev, flush):
         if name == "fwd_2step":
             d["units"] = "the deep units, two time steps per launch"
         kern[name] = d
-    del sim
-    return kern, {"n_steps": ws_.n_steps, "ms_per_time_step": step_ms}
+    return kern, {"n_steps": ws_.n_steps, "ms_per_time_step": step_ms, "step_forms": forms}
 
 
 def run_ours(args):
@@ -460,10 +491,7 @@ def run_ours(args):
     total_wall = max_over_ranks(sum(wall_s), ws, dev)
     t = sim.last_timing()
     gpu_launches = (t["fwd_launches"] + t["bwd_launches"] + 2) * args.steps
-    # small grids: two launches per forward step (the sampled pass below, one z group by
-    # name, runs and times the split half-steps)
-    direct_forward = (args.zgroups == 0 and args.forward < 1 and
-                      t["fwd_launches"] <= 2 * w.n_steps + w.n_steps // rec.k + 1)
+    forms = sim.step_forms()
     cell_updates = w.n_cells * w.n_steps
     value = job_rate(ws, cell_updates, args.steps, total_ms / 1e3)
 
@@ -475,7 +503,13 @@ def run_ours(args):
     r_ms = statistics.median(bwd_ms) / w.n_steps
     digest = B.kernel_digest()
     traffic = read_traffic(digest, args.workload)
-    kern, sampled = sampled_breakdown(A, fdtd, args, w, rec, dev, flush)
+
+    def sim_options(other):
+        apply_options(A, other, args)
+        if tuned:
+            autotune.apply(other, tuned["options"])
+
+    kern, sampled = sampled_breakdown(A, fdtd, args, w, rec, dev, flush, sim_options)
     per_launch = {"record": 1.0 / rec.k, "fwd_2step": 0.5}
     phases = {}
     for ph, ms in (("forward", f_ms), ("reverse", r_ms)):
@@ -519,10 +553,8 @@ def run_ours(args):
                    "parallelism": f"replicas x{ws}",
                    "l2": "state larger than L2; L2 also flushed before every timed step",
                    "zgroups": args.zgroups or "automatic",
-                   "forward_step": ("direct" if direct_forward else
-                                    "two steps per pass over the deep units" if "fwd_2step" in kern
-                                    else "fused" if "fwd_fused" in kern else "split"),
-                   "reverse_step": "fused" if "rev_primal" in kern else "split",
+                   "forward_step": STEP_LABELS[forms["forward"]],
+                   "reverse_step": STEP_LABELS[forms["reverse"]],
                    "autotuned": None if tuned is None else
                    {"options": tuned["options"], "cached": tuned["cached"]},
                    "fwd_ms": statistics.median(fwd_ms), "bwd_ms": statistics.median(bwd_ms),
@@ -586,8 +618,9 @@ def run_ours(args):
 # --------------------------------------------------------- profile run ---
 
 def run_profile(args):
-    """One short forward + backward with the given launch options (one launch
-    per half-step unless --zgroups says otherwise), for profilers."""
+    """One short forward + backward with the given launch options, for profilers: the
+    launches one after another (one z group) unless --zgroups says otherwise or a
+    direction runs the direct half-steps, which one z group by name would replace."""
     import torch
     from paper_2603_24027_gb300 import _capi as A
     from paper_2603_24027_gb300 import build as B
@@ -600,9 +633,9 @@ def run_profile(args):
         w = w.replace(pml_thickness=args.pml)
     rec = tape_cfg(A, args.tape)
     sim = fdtd.Simulation(w)
-    if args.zgroups == 0:
-        args.zgroups = 1
     apply_options(A, sim, args)
+    if args.zgroups == 0 and "direct" not in sim.step_forms().values():
+        sim.set_option(A.OPT_ZGROUPS, 1)
     sim.set_option(A.OPT_SAMPLE_EVERY, args.sample_every if args.sample_every != 50 else 0)
     eps = torch.from_numpy(w.eps).cuda()
     for _ in range(min(args.warmup, 1) + 1):

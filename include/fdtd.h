@@ -397,6 +397,14 @@ int fdtd_last_host_call_ms(const fdtd_handle* h, float* device_ms);
 
 /* ------------------------------------------------ introspection --------- */
 
+/* How the handle's time steps run with its present options (host only): what
+ * FDTD_OPT_FORWARD and FDTD_OPT_REVERSE resolve to, FDTD_STEP_DIRECT for the
+ * direct half-steps that only the automatic choice takes.  Kernel 0's
+ * half-steps count as split.  Sampled timing does not change the form; a group
+ * call may run a reverse that is direct here as split phases. */
+enum { FDTD_STEP_DIRECT = 0, FDTD_STEP_SPLIT = 1, FDTD_STEP_FUSED = 2, FDTD_STEP_TWO = 3 };
+int fdtd_step_forms(const fdtd_handle* h, int* forward, int* reverse);
+
 /* Host copies of the plan's tables (no device needed).  which: 0 b_E,
  * 1 a_E, 2 1/kappa_E (integer positions), 3 b_H, 4 a_H, 5 1/kappa_H
  * (half-integer positions); out has the axis length. */

@@ -34,6 +34,7 @@ K_FWD_H, K_FWD_E, K_RECORD, K_RESTORE, K_REV_E, K_REV_H, K_REV_PRIMAL, K_REV_ADJ
     K_REV_ADJOINT_CPML, K_FWD_FUSED, K_FWD_2STEP = range(12)
 KERNEL_NAMES = ["fwd_h", "fwd_e", "record", "restore_seed", "rev_e", "rev_h", "rev_primal",
                 "rev_adjoint", "monitor", "rev_adjoint_cpml", "fwd_fused", "fwd_2step"]
+STEP_FORMS = ["direct", "split", "fused", "two_step"]
 
 
 class Grid(C.Structure):
@@ -94,6 +95,7 @@ _PROTOS = {
                                      C.POINTER(RecordCfg), C.POINTER(C.c_double)]),
     "fdtd_batch_backward": (C.c_int, [C.POINTER(C.c_void_p), C.c_int, C.POINTER(C.c_double),
                                       C.POINTER(C.c_void_p)]),
+    "fdtd_step_forms": (C.c_int, [C.c_void_p, C.POINTER(C.c_int), C.POINTER(C.c_int)]),
     "fdtd_last_error": (C.c_char_p, [C.c_void_p]),
     "fdtd_destroy": (C.c_int, [C.c_void_p]),
     "fdtd_set_option": (C.c_int, [C.c_void_p, C.c_int, C.c_int]),

@@ -967,6 +967,19 @@ extern "C" int fdtd_get_option(const fdtd_handle* h, int option, int* value) {
 }
 
 // ------------------------------------------------------ introspection ---
+extern "C" int fdtd_step_forms(const fdtd_handle* h, int* forward, int* reverse) {
+  if (!h) return FDTD_EINVAL;
+  if (forward) {
+    const ForwardForm f = forward_form(h);
+    *forward = f == kDirect ? FDTD_STEP_DIRECT : f == kFusedStep ? FDTD_STEP_FUSED
+             : f == kTwoStep ? FDTD_STEP_TWO : FDTD_STEP_SPLIT;
+  }
+  if (reverse)
+    *reverse = direct_reverse(h) ? FDTD_STEP_DIRECT
+             : fused_reverse(h) ? FDTD_STEP_FUSED : FDTD_STEP_SPLIT;
+  return FDTD_OK;
+}
+
 extern "C" int fdtd_pml_profile(const fdtd_handle* h, int axis, int which, float* out) {
   if (!h || !out || axis < 0 || axis > 2 || which < 0 || which > 5) return FDTD_EINVAL;
   int n = axis == 0 ? h->nx : (axis == 1 ? h->ny : h->nz);

@@ -118,6 +118,13 @@ class Simulation:
         self._check(A.lib().fdtd_get_option(self.h, option, C.byref(v)))
         return v.value
 
+    def step_forms(self):
+        """How the time steps run with the present options: {"forward", "reverse"},
+        each "direct", "split", "fused" or (forward) "two_step"."""
+        f, r = C.c_int(), C.c_int()
+        self._check(A.lib().fdtd_step_forms(self.h, C.byref(f), C.byref(r)))
+        return {"forward": A.STEP_FORMS[f.value], "reverse": A.STEP_FORMS[r.value]}
+
     # -------------------------------------------------------------- runs ----
     @property
     def design_shape(self):
