@@ -1318,10 +1318,14 @@ struct ZGroups {
 };
 
 // Streams and events of the z-group scheduling of direction dir (created as
-// needed, outside a capture).
+// needed, outside a capture).  The fused steps use three of them for their side
+// launches, whatever the number of groups above one (two groups and a split forward
+// left the fused reverse with two streams and its four launches in a row: 137 against
+// 98 us per reverse step on 200 x 200 x 100, 234 against 195 on 301 x 203 x 151).
 static cudaError_t ensure_zgroups(fdtd_handle* h, int dir) {
   int want = zgroups_of(h, dir);
-  if (want > 1 && dir == 0 && forward_form(h) != kSplit) want = std::max(want, 3);
+  if (want > 1 && (dir == 0 ? forward_form(h) != kSplit : reverse_runs_fused(h)))
+    want = std::max(want, 3);
   if (want <= 1 || (int)h->zs.size() >= want) return cudaSuccess;
   cudaError_t e = cudaSuccess;
   if (!h->zfork) e = cudaEventCreateWithFlags(&h->zfork, cudaEventDisableTiming);
