@@ -41,6 +41,24 @@ def test_forms_by_grid(grid):
     assert (f["forward"], f["reverse"]) == GRIDS[grid]
 
 
+# Grids where the direct half-steps lose to the split ones below the general size line (every
+# warp meets an x slab) or keep winning there (tiles wasted): us per step in fdtd_api.cu.
+NARROW = {(64, 300, 135, 8): ("direct", "split"), (64, 300, 239, 8): ("split", "split"),
+          (64, 64, 292, 8): ("direct", "direct"), (64, 64, 463, 8): ("direct", "split"),
+          (64, 64, 1440, 8): ("split", "split"), (96, 96, 206, 12): ("direct", "split"),
+          (50, 200, 590, 8): ("split", "split"), (120, 120, 400, 8): ("split", "split"),
+          (160, 160, 230, 12): ("split", "split"), (160, 160, 74, 12): ("direct", "direct"),
+          (48, 48, 824, 8): ("direct", "direct"), (34, 34, 5103, 8): ("direct", "split"),
+          (600, 60, 163, 8): ("direct", "split"), (233, 181, 117, 12): ("direct", "split"),
+          (150, 110, 70, 12): ("direct", "direct")}
+
+
+@pytest.mark.parametrize("grid", NARROW)
+def test_forms_of_narrow_and_wide_grids(grid):
+    f = F.Simulation(problem(*grid)).step_forms()
+    assert (f["forward"], f["reverse"]) == NARROW[grid]
+
+
 def test_named_forms():
     sim = F.Simulation(problem(200, 200, 100, 6))
     for opt, val, key, form in ((A.OPT_FORWARD, 1, "forward", "split"),
