@@ -300,6 +300,7 @@ struct StepArgs {
   int zc0, zc1;     // two-cells-per-thread kernels: z chunks [zc0, zc1) of this launch (zc1 = 0: to the last)
   int zcs;          // two-step forward: planes per z chunk of U (the split half-steps' chunks)
   int t0x, t0y;     // fused reverse step: first tile of a launch along x and y
+  int overlap;      // fused reverse step: its launches run side by side
   int rows;         // the tile rows of a group of units, the planes [zb, ze) of the launch in
   int zb, ze, zl;   // chunks of zl, and the planes of the CPML-free units (all set by
   int zi0, zi1;     // launch_rev_fused)

@@ -44,7 +44,7 @@
 // 32-bit offset: 2071 -> 1974 us per reverse step (600 x 600 x 300), 671 -> 639
 // (411 x 389 x 203), 239 -> 218 (301 x 203 x 151).  A stream for each launch (in
 // fdtd_api.cu), the order of the units and the chunks' lengths (group_rows,
-// launch_chunk) took it to 1879, 602 and 194.
+// ring_chunk) took it to 1879, 602 and 194.
 #include <cudaTypedefs.h>
 
 #include "lag_common.cuh"
@@ -119,7 +119,7 @@ constexpr int adj_ctas() { return MODE == 2 ? 4 : (MODE == 1 ? 5 : 6); }
 // tiles [ix0, ix1) x [iy0, iy1) and the chunks outside [iz0, iz1)
 // (zonly_chunk).  Ring units (MODE 2): a 1D grid over every chunk times the
 // ring tiles (ring_unit).  A launch covers the planes [zb, ze) in chunks of zl
-// (launch_chunk).
+// (ring_chunk).
 //
 // Order of the primal and CPML-free launches (unit_order): groups of `rows` tile
 // rows, each with all its chunks before the next group.  A chunk reads two planes
@@ -144,15 +144,22 @@ inline int group_rows(dim3 grid) {
 }
 // Planes per chunk of a launch; zc: the chunk that the units are counted in.  Every
 // chunk streams two planes more than it owns, and a ring unit streams its
-// auxiliaries' and profiles' too: three times zc there (us per reverse step, ring
-// chunks of 8 / 24 / 32 / 64 planes: 1929 / 1893 / 1889 / 1884 on 600 x 600 x 300, 617 /
-// 609 / 608 / 611 on 411 x 389 x 203, 200 / 194 / 194 / 203 on 301 x 203 x 151, 151 /
-// 149 / 152 / - on 200 x 200 x 150, where one CTA's chain of planes begins to show).
+// auxiliaries' and profiles' too, so longer ring chunks move less; but a ring unit takes
+// 1.8 us a plane, and where the step's other launches are too short to hide that chain,
+// or run before and after it (overlap 0), it is the step.  us per reverse step, ring
+// chunks of 8 / 16 / 24 planes: 1929 / - / 1893 on 600 x 600 x 300 (32: 1889, 64: 1884), 617 /
+// - / 609 on 411 x 389 x 203, 201 / 198 / 195 on 301 x 203 x 151, 145 / 141 / 139 on 200 x 200 x
+// 150, 101 / 97 / 98 on 200 x 200 x 100, 65 / 63 / 75 on 200 x 200 x 60, 59 / 63 / 78 on 128^3,
+// 58 / 62 / 75 on 400 x 80 x 70, 31 / 43 / 60 on 100 x 100 x 50; one launch after another 230 /
+// 240 / 233 on 301 x 203 x 151, 125 / 123 / 137 on 200 x 200 x 100, 124 / 136 / 152 on 400 x 300 x
+// 40, 57 / 72 / 87 on 100 x 100 x 50.
 // The primal units take twice zc where they run in groups of tile rows (1887 -> 1878 on
 // 600 x 600 x 300, 893 -> 886 on 800 x 700 x 90; one group: no difference).  The
 // CPML-free adjoint units gain nothing (16 planes: 1927 against 1929; 24: 1967).
-inline int launch_chunk(int which, int zc, bool groups) {
-  return which == 3 ? 3 * zc : (which == 0 && groups ? 2 * zc : zc);
+inline int ring_chunk(const Geo& g, int zc, int overlap) {
+  const long long cells = (long long)g.nx * g.ny * g.nz;
+  const int planes = !overlap ? 0 : (cells >= 5000000 ? 24 : (cells >= 2400000 ? 16 : 0));
+  return zc * (planes >= 3 * zc ? 3 : (planes >= 2 * zc ? 2 : 1));
 }
 
 }  // namespace revf
@@ -925,13 +932,13 @@ cudaError_t launch_rev_fused(int which, const RevMaps& m, const StepArgs& a, con
       grid = dim3(U.px1 - U.px0, U.py1 - U.py0, 1);
       b.rows = group_rows(grid);
       grid.z = chunks(U.pz0 * zc, min(nz, U.pz1 * zc),
-                      launch_chunk(0, zc, b.rows < (int)grid.y));
+                      b.rows < (int)grid.y ? 2 * zc : zc);
       b.t0x = U.px0; b.t0y = U.py0;
       break;
     case 1:
       grid = dim3(U.ix1 - U.ix0, U.iy1 - U.iy0, 1);
       b.rows = group_rows(grid);
-      grid.z = chunks(b.zi0, b.zi1, launch_chunk(1, zc, false));
+      grid.z = chunks(b.zi0, b.zi1, zc);
       b.t0x = U.ix0; b.t0y = U.iy0;
       break;
     case 2:
@@ -940,7 +947,7 @@ cudaError_t launch_rev_fused(int which, const RevMaps& m, const StepArgs& a, con
       b.t0x = U.ix0; b.t0y = U.iy0;
       break;
     case 3:
-      grid = dim3((unsigned)(ring_tiles(U) * chunks(0, nz, launch_chunk(3, zc, false))), 1, 1);
+      grid = dim3((unsigned)(ring_tiles(U) * chunks(0, nz, ring_chunk(a.g, zc, a.overlap))), 1, 1);
       break;
     default:
       return cudaErrorInvalidValue;

@@ -34,3 +34,26 @@ def test_fused_reverse_launches_have_their_own_streams(run, zgroups, streams):
     rev = [e for e in log if e.what == "launch" and "k_rev_" in e.name]
     assert len(rev) == 4 * sim.w.n_steps
     assert len({e.a for e in rev}) == streams
+
+
+def ring_tiles(nx, ny, nz, P, zchunk):
+    """32 x 8 tiles that, with their neighbour cells, do not lie inside the x / y interior;
+    every tile where no unit (tile and z chunk) lies inside the interior."""
+    inside = [sum(t * w - 1 >= P and t * w + w < n - P for t in range(-(-n // w)))
+              for n, w in ((nx, 32), (ny, 8), (nz, zchunk or nz))]
+    box = inside[0] * inside[1] if inside[2] else 0
+    return -(-nx // 32) * -(-ny // 8) - box
+
+
+@pytest.mark.parametrize("grid,zgroups,zchunk,planes", [
+    ((100, 100, 50, 8), 0, 8, 8), ((128, 128, 128, 8), 0, 8, 8), ((200, 200, 100, 12), 0, 8, 16),
+    ((200, 200, 100, 12), 1, 8, 8), ((301, 203, 151, 10), 0, 8, 24), ((301, 203, 151, 10), 1, 8, 8),
+    ((301, 203, 151, 10), 0, 4, 12), ((301, 203, 151, 10), 0, 16, 16), ((301, 203, 151, 10), 0, 0, 151)])
+def test_ring_chunks_grow_where_other_launches_hide_them(run, grid, zgroups, zchunk, planes):
+    nx, ny, nz, P = grid
+    sim = run.sim(problem(*grid), REC, {A.OPT_REVERSE: 2, A.OPT_ZGROUPS: zgroups,
+                                        A.OPT_ZCHUNK: zchunk})
+    run.forward(sim, REC)
+    ring = [e.grid for e in run.backward(sim) if e.what == "launch" and "k_rev_adjoint" in e.name
+            and e.grid[1:] == (1, 1)]
+    assert ring and set(ring) == {(ring_tiles(nx, ny, nz, P, zchunk) * -(-nz // planes), 1, 1)}
