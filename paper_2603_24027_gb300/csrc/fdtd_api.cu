@@ -557,15 +557,21 @@ static bool direct_reverse(const fdtd_handle* h) {
 // 196 / 178 on 260 x 200 x 150, 224 / 194 (9.2 M), 717 / 602 (32 M).  An
 // option that names another shape of the split half-steps leaves the choice to the
 // units' CPML share alone.
+// With one z group (FDTD_OPT_ZGROUPS = 1) a pass and the other units' four launches
+// run in a row, each with a wave of CTAs that it does not fill; the line is higher then
+// (split / two steps: 142 / 200 on 301 x 203 x 151, 218 / 262 on 256^3, 250 / 289 on 301 x
+// 203 x 300 (18 M), 412 / 363 on 411 x 389 x 203, 469 / 416 on 600 x 600 x 100).
 enum ForwardForm { kSplit, kDirect, kFusedStep, kTwoStep };
-static const long long kFusedForwardCells = 12000000;
+static const long long kFusedForwardCells = 12000000, kTwoStepOneGroupCells = 24000000;
 static long long cells_of(const fdtd_handle* h) { return (long long)h->nx * h->ny * h->nz; }
+static bool two_step_pays(const fdtd_handle* h) {
+  if (h->opt_zgroups == 1) return cells_of(h) >= kTwoStepOneGroupCells;
+  return !direct_shape(h) || cells_of(h) >= kFusedForwardCells;
+}
 static ForwardForm forward_form(const fdtd_handle* h) {
   if (h->opt_kernel != 5 || h->opt_forward == 1) return kSplit;
   if (direct_forward(h)) return kDirect;
-  if (two_step_forward(h) && (h->opt_forward == 3 || !direct_shape(h) ||
-                              cells_of(h) >= kFusedForwardCells))
-    return kTwoStep;
+  if (two_step_forward(h) && (h->opt_forward == 3 || two_step_pays(h))) return kTwoStep;
   if (fused_forward(h) && (h->opt_forward == 2 || !direct_shape(h))) return kFusedStep;
   return h->opt_forward == 0 && direct_shape(h) && cells_of(h) >= kFusedForwardCells ? kFusedStep
                                                                                      : kSplit;

@@ -70,6 +70,17 @@ def test_named_forms():
         assert sim.step_forms()[key] == form
 
 
+@pytest.mark.parametrize("grid,form", [((400, 80, 70, 4), "split"), ((301, 203, 151, 10), "split"),
+                                       ((256, 256, 256, 8), "split"),
+                                       ((411, 389, 203, 10), "two_step")])
+def test_one_z_group_runs_two_steps_per_pass_on_large_grids_only(grid, form):
+    sim = F.Simulation(problem(*grid))
+    sim.set_option(A.OPT_ZGROUPS, 1)
+    assert sim.step_forms()["forward"] == form
+    sim.set_option(A.OPT_FORWARD, 3)
+    assert sim.step_forms()["forward"] == "two_step"
+
+
 @pytest.mark.parametrize("inside", [False, True])
 @pytest.mark.parametrize("grid", GRIDS)
 def test_sampled_runs_time_the_forms_of_the_timed_run(grid, inside):
