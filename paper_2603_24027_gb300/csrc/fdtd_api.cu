@@ -42,7 +42,7 @@ struct Layout {
 struct GraphKey {
   int dir, dtype, k, interp, scaled, kernel, tile_y, zchunk, sample, stages, pdl, prefetch,
       tile_x, compact, exact, coeffs, zchunk_fwd, zgroups, inject_wait, reverse, forward,
-      zchunk_fwd2, start_buf, group_split;
+      zchunk_fwd2, start_buf, grouped;
   bool operator<(const GraphKey& o) const {
     return memcmp(this, &o, sizeof(GraphKey)) < 0;
   }
@@ -86,6 +86,7 @@ struct fdtd_handle {
   size_t ws_bytes;
   bool tables_uploaded;
   bool group_split;           // this loop of a group call takes the split reverse phases
+  bool group_two;             // this loop of a group call takes two steps per pass, if it may
   bool one_stream;            // the no-allocation call: every launch on the caller's stream
   bool have_forward;
   int fwd_buf;                // field buffer holding the state after forward
@@ -566,7 +567,7 @@ static const long long kFusedForwardCells = 12000000, kTwoStepOneGroupCells = 24
 static long long cells_of(const fdtd_handle* h) { return (long long)h->nx * h->ny * h->nz; }
 static bool two_step_pays(const fdtd_handle* h) {
   if (h->opt_zgroups == 1) return cells_of(h) >= kTwoStepOneGroupCells;
-  return !direct_shape(h) || cells_of(h) >= kFusedForwardCells;
+  return !direct_shape(h) || h->group_two || cells_of(h) >= kFusedForwardCells;
 }
 static ForwardForm forward_form(const fdtd_handle* h) {
   if (h->opt_kernel != 5 || h->opt_forward == 1) return kSplit;
@@ -799,6 +800,7 @@ extern "C" int fdtd_create(const fdtd_grid* grid, double dx, double dt, const fd
   h->opt_zgroups = 0;
   h->one_stream = false;
   h->group_split = false;
+  h->group_two = false;
   h->zfork = nullptr;
   h->opt_sample = 0;
   h->opt_stages = 2;
@@ -1877,7 +1879,7 @@ static int run_loop(fdtd_handle* h, const fdtd_record_cfg* rec, int dir, Enqueue
   key.reverse = h->opt_reverse;
   key.forward = h->opt_forward;
   key.zchunk_fwd2 = h->opt_zchunk_fwd2;
-  key.group_split = dir == 1 && h->group_split;
+  key.grouped = dir == 1 ? h->group_split : h->group_two;
   key.start_buf = dir == 1 ? h->fwd_buf : 0;   // the backward starts from the forward's buffer
   auto it = h->graphs.find(key);
   if (it == h->graphs.end()) {
@@ -2157,10 +2159,21 @@ extern "C" int fdtd_value_and_grad_host(fdtd_handle* h, const float* h_eps,
 // left.  ms for twenty cubes of 48^3 to 128^3 / sixty-four of 32^3 to 128^3: 30.5 / 732
 // with 0.6 of the cache, 33.5 / 735 with 0.3, 31.6 / 691 with 1.0, 35.1 / 784 with 2, 35.5
 // / 811 all at once.
-static const double kGroupCacheShare = 0.6;
+//
+// A state well above the cache (kGroupNoCache of it) comes from HBM whether its loop
+// runs alone or not: such loops start at once.  Several of them together are bound by
+// the bytes they move, so those that may run two steps per pass do, also below the
+// size from which a single one does.  Small loops run beside them; one that needs most
+// of the cache waits until they are done, after the small ones.  ms, one after
+// another / side by side / side by side with two steps per pass: four of 301 x 203 x 151
+// 20.4 / 19.9 / 17.4, of 300 x 300 x 120 - / 22.5 / 19.1, of 400 x 300 x 90 - / 22.4 / 17.7, of 300 x
+// 300 x 150 (two steps in any case) 25.5 / - / 24.0; four of 200 x 200 x 100 (1.08 of the cache)
+// 13.4 / 14.0 / -, three of 160^3 10.8 / 11.2 / -.
+static const double kGroupCacheShare = 0.6, kGroupNoCache = 1.6;
 struct GroupSlot {
   int i;                    // index in the call
   std::vector<int> after;   // indices of the loops it waits for
+  bool two;                 // two steps per pass where the grid may
 };
 static std::vector<GroupSlot> group_plan(fdtd_handle* const* hs, int n) {
   int dev = 0, l2 = 0;
@@ -2168,8 +2181,9 @@ static std::vector<GroupSlot> group_plan(fdtd_handle* const* hs, int n) {
       cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess || l2 <= 0)
     l2 = 128 << 20;
   const double room = kGroupCacheShare * l2;
-  struct Loop { int i; double bytes, seconds; };
+  struct Loop { int i; double bytes, seconds; bool alone; };
   std::vector<Loop> todo;
+  std::vector<GroupSlot> plan;
   for (int i = 0; i < n; ++i) {
     const fdtd_handle* h = hs[i];
     const double nc = (double)cells_of(h);
@@ -2177,13 +2191,22 @@ static std::vector<GroupSlot> group_plan(fdtd_handle* const* hs, int n) {
     // measured: seconds a step and a cell and step
     const double step = direct_forward(h) ? 4.5e-6 + 8.5e-12 * nc : 15e-12 * nc;
     const double bytes = 28.0 * nc + psi;
-    todo.push_back({i, std::min(bytes, 0.8 * room), step * h->N});
+    if (bytes > kGroupNoCache * l2)
+      plan.push_back({i, {}, true});
+    else
+      todo.push_back({i, std::min(bytes, 0.8 * room), step * h->N, bytes > room});
   }
-  std::stable_sort(todo.begin(), todo.end(),
-                   [](const Loop& a, const Loop& b) { return a.bytes > b.bytes; });
+  std::vector<int> first;   // the loops above the cache
+  for (GroupSlot& s : plan) {
+    s.two = plan.size() > 1;
+    first.push_back(s.i);
+  }
+  std::stable_sort(todo.begin(), todo.end(), [&](const Loop& a, const Loop& b) {
+    if (!first.empty() && a.alone != b.alone) return b.alone;
+    return a.bytes > b.bytes;
+  });
   struct Run { double end, bytes; int i; };
   std::vector<Run> running;
-  std::vector<GroupSlot> plan;
   std::vector<int> freed;   // the loops whose end made the room there is now
   double now = 0.0, used = 0.0;
   while (!todo.empty()) {
@@ -2194,7 +2217,9 @@ static std::vector<GroupSlot> group_plan(fdtd_handle* const* hs, int n) {
       }
       running.push_back({now + todo[t].seconds, todo[t].bytes, todo[t].i});
       used += todo[t].bytes;
-      plan.push_back({todo[t].i, freed});
+      plan.push_back({todo[t].i, freed, false});
+      if (todo[t].alone)
+        plan.back().after.insert(plan.back().after.end(), first.begin(), first.end());
       todo.erase(todo.begin() + t);
     }
     if (todo.empty()) break;
@@ -2229,7 +2254,9 @@ extern "C" int fdtd_group_forward(fdtd_handle* const* hs, int n, const float* co
   }
   for (const GroupSlot& s : group_plan(hs, n)) {
     int rc = group_wait(hs, s);
+    hs[s.i]->group_two = s.two;
     if (!rc) rc = forward_async(hs[s.i], d_eps[s.i], rec);
+    hs[s.i]->group_two = false;
     if (rc) return rc;
   }
   for (int i = 0; i < n; ++i) {

@@ -57,3 +57,48 @@ def test_ring_chunks_grow_where_other_launches_hide_them(run, grid, zgroups, zch
     ring = [e.grid for e in run.backward(sim) if e.what == "launch" and "k_rev_adjoint" in e.name
             and e.grid[1:] == (1, 1)]
     assert ring and set(ring) == {(ring_tiles(nx, ny, nz, P, zchunk) * -(-nz // planes), 1, 1)}
+
+
+def waits_of(log, sims, run):
+    """Per simulation the set of simulations whose loops its own loop waits for: the
+    events of the other loops' ends that its stream waits for before its launches."""
+    stream, end = {}, {}
+    loops = [e.a for e in log if e.what == "graph"]
+    for s in loops:                      # the record right after a loop's graph is its end
+        at = next(i for i, e in enumerate(log) if e.what == "graph" and e.a == s)
+        end[next(e.b for e in log[at:] if e.what == "record" and e.a == s)] = s
+    out = {s: set() for s in loops}
+    for e in log:
+        if e.what == "wait" and e.b in end and e.a in out:
+            out[e.a].add(end[e.b])
+    return loops, out
+
+
+LARGE, MID, SMALL = (301, 203, 151, 10), (200, 200, 100, 12), (64, 64, 64, 8)
+
+
+@pytest.mark.parametrize("grids,free", [([LARGE] * 4, 4), ([MID] * 3, 1), ([LARGE, MID, MID], 1),
+                                        ([SMALL] * 6, 5), ([LARGE] + [SMALL] * 3, 4),
+                                        ([MID] + [SMALL] * 3, 2)])
+def test_group_forward_waits_only_for_states_that_share_the_cache(run, grids, free):
+    """Loops whose state no cache holds start at once; of those that nearly fill it one
+    runs at a time, after the former; small ones fit beside each other.  Room
+    for 0.6 of 132.6 MB: five states of 64^3 (28 bytes a cell, x auxiliaries of the whole
+    grid, compact ones along y and z: 13.6 MB), or one that counts as 0.8 of it and one."""
+    sims = [run.sim(problem(*g), REC) for g in grids]
+    loops, waits = waits_of(run.group_forward(sims, REC), sims, run)
+    assert len(loops) == len(grids)
+    assert sum(not w for w in waits.values()) == free
+    started = []
+    for s in loops:                      # only loops that are enqueued already
+        assert waits[s] <= set(started)
+        started.append(s)
+
+
+@pytest.mark.parametrize("grids,two", [([LARGE], 0), ([LARGE, LARGE], 2), ([LARGE, MID], 0), ([LARGE, LARGE, MID], 2),
+                                       ([LARGE] + [SMALL] * 3, 0), ([MID, MID], 0)])
+def test_large_loops_of_a_group_run_two_steps_per_pass(run, grids, two):
+    sims = [run.sim(problem(*g), REC) for g in grids]
+    log = run.group_forward(sims, REC)
+    assert len({e.a for e in log if e.what == "launch" and "k_fwd_2step" in e.name}) == two
+    assert all(s.step_forms()["forward"] != "two_step" for s in sims)
