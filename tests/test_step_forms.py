@@ -49,7 +49,7 @@ NARROW = {(64, 300, 135, 8): ("direct", "split"), (64, 300, 239, 8): ("split", "
           (50, 200, 590, 8): ("split", "split"), (120, 120, 400, 8): ("split", "split"),
           (160, 160, 230, 12): ("split", "split"), (160, 160, 74, 12): ("direct", "direct"),
           (48, 48, 824, 8): ("direct", "direct"), (34, 34, 5103, 8): ("direct", "split"),
-          (600, 60, 163, 8): ("direct", "split"), (233, 181, 117, 12): ("direct", "split"),
+          (600, 60, 163, 8): ("direct", "split"), (400, 300, 50, 8): ("direct", "split"), (233, 181, 117, 12): ("direct", "split"),
           (150, 110, 70, 12): ("direct", "direct")}
 
 
