@@ -2252,6 +2252,12 @@ extern "C" int fdtd_group_forward(fdtd_handle* const* hs, int n, const float* co
     int rc = forward_check(hs[i], d_eps[i], rec);
     if (rc) return rc;
   }
+  // A first call uploads a handle's tables and waits for them: before any stream waits
+  // for another loop, or the host would wait for that loop too and enqueue the rest late.
+  for (int i = 0; i < n; ++i) {
+    int rc = begin(hs[i]);
+    if (rc) return rc;
+  }
   for (const GroupSlot& s : group_plan(hs, n)) {
     int rc = group_wait(hs, s);
     hs[s.i]->group_two = s.two;

@@ -102,3 +102,14 @@ def test_large_loops_of_a_group_run_two_steps_per_pass(run, grids, two):
     log = run.group_forward(sims, REC)
     assert len({e.a for e in log if e.what == "launch" and "k_fwd_2step" in e.name}) == two
     assert all(s.step_forms()["forward"] != "two_step" for s in sims)
+
+
+def test_first_group_forward_blocks_the_host_for_no_loop(run):
+    """Every member's tables are uploaded (the host waits for the copies) before a stream
+    waits for another loop's end; after that the host waits for results only."""
+    sims = [run.sim(problem(*g), REC) for g in (MID, MID, MID, SMALL)]
+    log = run.group_forward(sims, REC)
+    what = [e.what for e in log]
+    first, last = what.index("graph"), len(what) - 1 - what[::-1].index("graph")
+    assert what.count("graph") == 4
+    assert what[:first].count("sync") == 4 and "sync" not in what[first:last]
