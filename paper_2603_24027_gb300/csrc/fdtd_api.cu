@@ -2049,6 +2049,8 @@ static int backward_async(fdtd_handle* h, double seed, double seed2) {
   rc = begin(h);
   if (rc) return rc;
   CK(h, upload_seeds(h, layout_of(h, &h->fwd_rec), seed, seed2, h->stream));
+  // the forward may have run in another process (fdtd_load_state)
+  if (h->fwd_rec.dtype == kTapeBdct) CK(h, bdct_ensure_basis());
   int nl = 0;
   nvtxRangePushA("fdtd backward loop");
   rc = run_loop(h, &h->fwd_rec, 1, enqueue_backward, &nl, h->t2, h->t3);

@@ -113,3 +113,24 @@ def test_first_group_forward_blocks_the_host_for_no_loop(run):
     first, last = what.index("graph"), len(what) - 1 - what[::-1].index("graph")
     assert what.count("graph") == 4
     assert what[:first].count("sync") == 4 and "sync" not in what[first:last]
+
+
+def test_backward_from_a_loaded_state_uploads_the_block_codecs_basis(tmp_path, monkeypatch):
+    """A process that only loads a saved forward and runs the backward decodes a block
+    codec tape with the basis table, which no forward of its own has uploaded."""
+    import ctypes as C
+    w, rec = problem(*SMALL), A.record_cfg("bdct10", 2)
+    saver = S.Runner(S.load(tmp_path), monkeypatch)
+    sim = saver.sim(w, rec)
+    saver.forward(sim, rec)
+    n = C.c_size_t()
+    A.check(saver.L.fdtd_state_bytes(sim.h, C.byref(n)), sim.h)
+    blob = C.create_string_buffer(n.value)
+    A.check(saver.L.fdtd_save_state(sim.h, blob, n.value), sim.h)
+    sim.close()
+    (tmp_path / "other").mkdir()
+    loader = S.Runner(S.load(tmp_path / "other"), monkeypatch)   # a library not used before
+    sim = loader.sim(w, rec)
+    A.check(loader.L.fdtd_load_state(sim.h, blob, n.value), sim.h)
+    what = [e.what for e in loader.backward(sim)]
+    assert what.count("symbol") == 2 and what.index("symbol") < what.index("launch")
