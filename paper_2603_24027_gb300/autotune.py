@@ -11,8 +11,14 @@ grid, CPML, source, detector, design box, tape and kernel; fewer time steps),
 searching one option at a time from the current settings (coordinate
 descent, repeated until a pass changes nothing), applies the fastest to the
 simulation and stores it in a JSON cache keyed by the GPU name, the grid,
-the CPML thickness, the kernel and the tape configuration, so that a
-problem of the same shape is tuned once per GPU type.
+the CPML thickness, the kernel, the tape configuration and the library's
+sources, so that a problem of the same shape is tuned once per GPU type and
+build.
+
+On a grid whose steps run as direct half-steps any value but the default of
+z groups, z chunk, forward z chunk, tile height or stages names a shape of the
+split half-steps and takes the grid off the direct ones; the search starts
+from the defaults and keeps them there unless a split shape is faster.
 
     from paper_2603_24027_gb300 import autotune
     best = autotune.tune(sim, eps, rec)          # times, applies, caches
@@ -30,6 +36,7 @@ import time
 from typing import Callable, Dict, Iterable, List, Optional, Sequence, Tuple
 
 from . import _capi as A
+from . import build as B
 
 # option name -> (library option id, candidate values in the order tried)
 SPACE: List[Tuple[str, int, Sequence[int]]] = [
@@ -56,8 +63,10 @@ def default_cache_path() -> str:
 
 
 def cache_key(gpu_name: str, workload, kernel: int, rec) -> str:
-    """GPU type, grid, CPML thickness, kernel and tape configuration."""
-    return (f"{gpu_name}|{workload.nx}x{workload.ny}x{workload.nz}|P{workload.pml_thickness}"
+    """GPU type, grid, CPML thickness, kernel, tape configuration and the library's
+    sources (an entry of another build names shapes that build ran best, which on a grid
+    with a form of step that it lacked is the slower choice)."""
+    return (f"{B.source_digest()}|{gpu_name}|{workload.nx}x{workload.ny}x{workload.nz}|P{workload.pml_thickness}"
             f"|kernel{kernel}|tape{rec.dtype}:{rec.k}:{rec.interp}:{rec.scaled}:{rec.coeffs}")
 
 

@@ -44,6 +44,19 @@ def _digest() -> str:
     return h.hexdigest()[:16]
 
 
+def source_digest() -> str:
+    """Digest of the library's sources and compile flags without the include path, so
+    that copies of the tree at other paths (and machines) agree."""
+    h = hashlib.sha256()
+    for name in sorted(os.listdir(CSRC)):
+        with open(os.path.join(CSRC, name), "rb") as f:
+            h.update(name.encode() + f.read())
+    with open(os.path.join(INCLUDE, "fdtd.h"), "rb") as f:
+        h.update(f.read())
+    h.update(" ".join(ARCH + [x for x in FLAGS if not x.startswith("-I")]).encode())
+    return h.hexdigest()[:16]
+
+
 # Device code of the default half-step kernels: the files whose change can
 # change what those kernels move through memory.
 KERNEL_FILES = ["kernels_lag2.cu", "kernels_rev_fused.cu", "kernels_fwd_fused.cu",
