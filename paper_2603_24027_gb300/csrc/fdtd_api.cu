@@ -516,8 +516,8 @@ static const long long kDirectForwardCells = 6000000, kDirectReverseCells = 2000
 // that meets an x slab loads and stores its auxiliaries too, for as long as the whole
 // warp: of rows of 32 pairs every warp does, of rows of 300 one in eight.  The staged
 // kernels lose what their 32 x 8 tiles cover beyond the plane.  So the cells, times 1 +
-// the share of such warps, are held against `limit` times the tiles' waste to the
-// power 3/2.  us per step, direct against split: forward on 64 x 300 x 135 cells (every warp
+// 0.8 of the square of such warps' share, are held against `limit` times the tiles' waste
+// to the power 3/2 (the powers that fit both directions' figures).  us per step, direct against split: forward on 64 x 300 x 135 cells (every warp
 // meets a slab, no waste) 41.8 / 45.2, x 182 58.9 / 58.2, x 307 105 / 92; 96 x 96 x 379 53.0 /
 // 52.8, x 640 93 / 85; 160 x 160 x 136 (half the warps) 48.5 / 50.2, x 230 86 / 81; 48 x 48 x 1996
 // (every warp, waste 1.33) 84.5 / 85.7, x 2560 111 / 108; 34 x 34 x 5103 (waste 1.66) 144 / 156;
@@ -528,7 +528,7 @@ static bool direct_pays(const fdtd_handle* h, double limit) {
   const int pairs = h->px / 2;   // of a row
   const double share = std::min(1.0, (h->P + 31.0) / pairs);
   const double waste = up(h->nx, 32) * up(h->ny, 8) / (2.0 * up(pairs * h->ny, 128));
-  return (double)h->nx * h->ny * h->nz * (1.0 + share) <= limit * waste * sqrt(waste);
+  return (double)h->nx * h->ny * h->nz * (1.0 + 0.8 * share * share) <= limit * waste * sqrt(waste);
 }
 static bool direct_shape(const fdtd_handle* h) {
   return h->opt_kernel == 5 && h->opt_tile_y == 8 && h->opt_tile_x == 32 && h->opt_stages == 2 &&
@@ -538,11 +538,11 @@ static bool direct_shape(const fdtd_handle* h) {
 static Geo geo_of(const fdtd_handle* h);
 static bool direct_forward(const fdtd_handle* h) {
   return direct_shape(h) && direct_fits(geo_of(h)) && h->opt_forward == 0 &&
-         (long long)h->nx * h->ny * h->nz <= kDirectForwardCells && direct_pays(h, 6.8e6);
+         (long long)h->nx * h->ny * h->nz <= kDirectForwardCells && direct_pays(h, 6.2e6);
 }
 static bool direct_reverse(const fdtd_handle* h) {
   return !h->group_split && direct_shape(h) && direct_fits(geo_of(h)) && h->opt_reverse == 0 &&
-         (long long)h->nx * h->ny * h->nz <= kDirectReverseCells && direct_pays(h, 3.05e6);
+         (long long)h->nx * h->ny * h->nz <= kDirectReverseCells && direct_pays(h, 2.8e6);
 }
 
 // How a forward and a reverse run.  Named forms (FDTD_OPT_FORWARD 1-3,
