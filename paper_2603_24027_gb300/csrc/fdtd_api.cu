@@ -2163,14 +2163,17 @@ extern "C" int fdtd_value_and_grad_host(fdtd_handle* h, const float* h_eps,
 // / 811 all at once.
 //
 // A state well above the cache (kGroupNoCache of it) comes from HBM whether its loop
-// runs alone or not: such loops start at once.  Several of them together are bound by
-// the bytes they move, so those that may run two steps per pass do, also below the
-// size from which a single one does.  Small loops run beside them; one that needs most
-// of the cache waits until they are done, after the small ones.  ms, one after
-// another / side by side / side by side with two steps per pass: four of 301 x 203 x 151
-// 20.4 / 19.9 / 17.4, of 300 x 300 x 120 - / 22.5 / 19.1, of 400 x 300 x 90 - / 22.4 / 17.7, of 300 x
-// 300 x 150 (two steps in any case) 25.5 / - / 24.0; four of 200 x 200 x 100 (1.08 of the cache)
-// 13.4 / 14.0 / -, three of 160^3 10.8 / 11.2 / -.
+// runs alone or not, and so does most of one that needs more than its share and runs
+// other forms than the direct half-steps (ms for four of 200 x 200 x 100 as split
+// half-steps, one after another / side by side: 14.5 / 14.2): such loops start at once.
+// Several above the cache together are bound by the bytes they move, so those that may
+// run two steps per pass do, also below the size from which a single one does.  Small
+// loops run beside them; a direct one that needs most of the cache waits until they are
+// done, after the small ones.  ms, one after another / side by side / side by side with
+// two steps per pass: four of 301 x 203 x 151 20.4 / 19.9 / 17.3, of 300 x 300 x 120 - / 22.5 /
+// 19.1, of 400 x 300 x 90 - / 22.4 / 17.7, of 300 x 300 x 150 (two steps in any case) 25.5 / - /
+// 24.0; four of 200 x 200 x 100 (1.08 of the cache, direct) 13.4 / 14.0 / -, three of 160^3 10.8 /
+// 11.2 / -.
 static const double kGroupCacheShare = 0.6, kGroupNoCache = 1.6;
 struct GroupSlot {
   int i;                    // index in the call
@@ -2193,14 +2196,15 @@ static std::vector<GroupSlot> group_plan(fdtd_handle* const* hs, int n) {
     // measured: seconds a step and a cell and step
     const double step = direct_forward(h) ? 4.5e-6 + 8.5e-12 * nc : 15e-12 * nc;
     const double bytes = 28.0 * nc + psi;
-    if (bytes > kGroupNoCache * l2)
-      plan.push_back({i, {}, true});
+    const bool above = bytes > kGroupNoCache * l2;
+    if (above || (bytes > room && !direct_forward(h)))
+      plan.push_back({i, {}, above});
     else
       todo.push_back({i, std::min(bytes, 0.8 * room), step * h->N, bytes > room});
   }
-  std::vector<int> first;   // the loops above the cache
+  std::vector<int> first;   // the loops that the cache does not serve
   for (GroupSlot& s : plan) {
-    s.two = plan.size() > 1;
+    s.two = s.two && plan.size() > 1;
     first.push_back(s.i);
   }
   std::stable_sort(todo.begin(), todo.end(), [&](const Loop& a, const Loop& b) {

@@ -95,6 +95,12 @@ def test_group_forward_waits_only_for_states_that_share_the_cache(run, grids, fr
         started.append(s)
 
 
+def test_group_forward_of_split_loops_that_fill_the_cache_runs_side_by_side(run):
+    sims = [run.sim(problem(*MID), REC, {A.OPT_FORWARD: 1}) for _ in range(3)]
+    _, waits = waits_of(run.group_forward(sims, REC), sims, run)
+    assert not any(waits.values()) and len(waits) == 3
+
+
 @pytest.mark.parametrize("grids,two", [([LARGE], 0), ([LARGE, LARGE], 2), ([LARGE, MID], 0), ([LARGE, LARGE, MID], 2),
                                        ([LARGE] + [SMALL] * 3, 0), ([MID, MID], 0)])
 def test_large_loops_of_a_group_run_two_steps_per_pass(run, grids, two):
