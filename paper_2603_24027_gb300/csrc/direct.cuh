@@ -38,7 +38,7 @@ struct DirectArgs {
   BdctLayout bl;       // block codec: its sample layout and basis table (device)
   const float* beta;
   void* tape;          // forward: the sample; reverse: the tape
-  long long stride;
+  long long stride;    // elements of a sample
   float* scale_slot;   // forward: the sample's scales
   const float* scales;
   Interp ip;

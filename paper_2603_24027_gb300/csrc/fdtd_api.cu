@@ -1427,6 +1427,7 @@ static cudaError_t enqueue_forward(fdtd_handle* h, const fdtd_record_cfg* rec, i
     d.psiA = a.psiA;
     d.F = a.F;
     d.tdtype = rec->dtype;
+    d.stride = L.stride;
     if (fold) d.det2 = det2;
     for (int n = 0; n < h->N; ++n) {
       const bool rec_now = n >= r && (n - r) % rec->k == 0;

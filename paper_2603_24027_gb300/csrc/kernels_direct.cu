@@ -201,6 +201,12 @@ __device__ __forceinline__ void record_side(const DirectArgs& a, int side, int r
   const long long q = face_value_cell(a.g, fd, rr, &comp);
   const float x = a.F[comp * a.g.nc + q];
   const long long o = fd.off + rr;
+#ifdef FDTD_BOUNDS_CHECK
+  if (o < 0 || o >= a.stride) {   // one sample's values
+    atomicOr(a.err, ERR_BOUNDS);
+    return;
+  }
+#endif
   switch (a.tdtype) {
     case 0: reinterpret_cast<Code<0>::T*>(a.tape)[o] = Code<0>::enc(x); break;
     case 1: reinterpret_cast<Code<1>::T*>(a.tape)[o] = Code<1>::enc(x); break;
@@ -257,6 +263,9 @@ __device__ __forceinline__ void restore_side(const DirectArgs& a, int side, int 
   }
   int comp;
   const long long q = face_value_cell(a.g, fd, rr, &comp);
+#ifdef FDTD_BOUNDS_CHECK
+  if (!store_ok(a, a.F + comp * a.g.nc + q)) return;
+#endif
   a.F[comp * a.g.nc + q] = val;
 }
 
