@@ -1,6 +1,6 @@
-// lag_common.cuh -- pieces shared by the one-plane-per-iteration kernels
-// (one and two x-cells per thread): CPML helpers, the plane ring, box
-// geometry and the shared-memory stage layout of each half-step.
+// lag_common.cuh -- pieces shared by the one-plane-per-iteration kernels: CPML
+// helpers, the plane ring, box geometry and the shared-memory stage layout of each
+// half-step.
 #pragma once
 
 #include "fdtd_internal.cuh"
@@ -12,20 +12,6 @@ namespace lag {
 
 constexpr int r128(int b) { return (b + 127) / 128 * 128; }
 
-__device__ __forceinline__ float cpml_s(float d, float psi_old, float* pout, long long pi, float b,
-                                        float a, float kv) {
-  float s = __fmaf_rn(b, psi_old, __fmul_rn(a, d));
-  pout[pi] = s;
-  return __fmaf_rn(kv, d, s);
-}
-
-__device__ __forceinline__ float adj_s(float v, float lpsi, float* pout, long long pi, bool own,
-                                       float b, float a, float kv) {
-  float mu = lpsi + v;
-  if (own) pout[pi] = b * mu;
-  return kv * v + a * mu;
-}
-
 __device__ __forceinline__ float src_wt(const Src& s, int i, int j, int k) {
   int u, v;
   if (s.kind == 0 || !on_plane(s.axis, s.index, s.u0, s.u1, s.v0, s.v1, i, j, k, &u, &v))
@@ -35,45 +21,6 @@ __device__ __forceinline__ float src_wt(const Src& s, int i, int j, int k) {
 
 __device__ __forceinline__ bool tile_in_slab(int lo, int hi_incl, int n, int P) {
   return lo < P || hi_incl >= n - P;
-}
-
-// Ring over planes p0..p1 (see kernels_split_tma.cu): plane p in stage
-// (p - p0) % S, barrier parity ((p - p0) / S) & 1.  Here every plane is read
-// in exactly one iteration, after which its stage is re-armed for p + S.
-template <int S>
-struct Ring {
-  unsigned char* base;
-  uint64_t* bars;
-  int stage_bytes, p0, p1;
-  __device__ unsigned char* at(int p) const { return base + ((p - p0) % S) * stage_bytes; }
-  __device__ uint64_t* bar(int p) const { return &bars[(p - p0) % S]; }
-  __device__ bool wait(int p) const {
-    return mbar_wait(bar(p), ((p - p0) / S) & 1, kWaitCycles);
-  }
-};
-
-template <int S>
-__device__ __forceinline__ Ring<S> ring_setup(unsigned char* dsm, int stage_bytes, int p0, int p1) {
-  Ring<S> r;
-  r.base = dsm;
-  r.bars = reinterpret_cast<uint64_t*>(dsm + S * stage_bytes);
-  r.stage_bytes = stage_bytes;
-  r.p0 = p0;
-  r.p1 = p1;
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
-    for (int s = 0; s < S; ++s) mbar_init(&r.bars[s], 1);
-    mbar_fence_init();
-  }
-  __syncthreads();
-  return r;
-}
-
-template <int S>
-__device__ void ring_drain(const Ring<S>& r, int p_waited, unsigned* err) {
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
-    atomicOr(err, ERR_TIMEOUT);
-    for (int p = p_waited; p <= r.p1 && p < p_waited + S; ++p) r.wait(p);
-  }
 }
 
 // Box geometry of a TW x TY tile: "lo" boxes start at (x0-4, y0-1) and cover
@@ -161,9 +108,10 @@ __device__ __forceinline__ float cpml(float d, float psi_old, float b, float a, 
 }
 
 // Adjoint of the recursion: returns the curl term with the CPML response.  The
-// adjoint's products and sums are rounded explicitly, in the same order in every
-// kernel, so that its fields and the gradient do not depend on which kernels run;
-// the adjoint auxiliary for the next (earlier) step goes to *out.
+// adjoint's products and sums are rounded explicitly, in the same order in the staged,
+// fused and direct kernels, so that its fields and the gradient do not depend on which of
+// them run (kernel 0, the plain-load cross-check, leaves its own to the compiler); the
+// adjoint auxiliary for the next (earlier) step goes to *out.
 __device__ __forceinline__ float adj(float v, float lpsi, float b, float a, float kv, float* out) {
   const float mu = lpsi + v;
   *out = b * mu;
