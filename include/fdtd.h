@@ -193,9 +193,10 @@ int fdtd_value_and_grad_host(fdtd_handle* h, const float* h_eps, const fdtd_reco
 /* Batched designs: n independent handles (each with its own workspace)
  * processed together; objs[i] / d_grads[i] as in fdtd_forward/backward.
  * Each handle runs its own time loop (a CUDA graph on its own stream); all
- * are enqueued before any is awaited.  The forwards run concurrently as far as
- * their states share the L2 cache, the others waiting on the device for room;
- * the backwards all run concurrently. */
+ * are enqueued before any is awaited.  The forwards of grids whose state the L2
+ * cache can hold run concurrently as far as their states share it, the others
+ * waiting on the device for room; larger grids' forwards, and all backwards, run
+ * concurrently. */
 int fdtd_group_forward(fdtd_handle* const* hs, int n, const float* const* d_eps,
                        const fdtd_record_cfg* rec, double* objs);
 int fdtd_group_backward(fdtd_handle* const* hs, int n, const double* seeds,
@@ -213,9 +214,10 @@ int fdtd_group_backward(fdtd_handle* const* hs, int n, const double* seeds,
  * once into CUDA graphs; the plan (tables and graphs, allocated by the
  * library with cudaMalloc, outside the time loops) belongs to hs[0] and is
  * rebuilt when the list, a workspace or an option changes; it is freed with
- * hs[0].  Every handle must run kernel 5's split steps (FDTD_OPT_FORWARD and
- * FDTD_OPT_REVERSE resolving to 1) with 32 x 8 tiles and two stages, one
- * detector, no exact reversal, and an unscaled tape format; else
+ * hs[0].  The steps are kernel 5's split half-steps.  Every handle must be one
+ * that may run them here: 32 x 8 tiles and two stages, neither the fused nor
+ * the two-step form named or open to the automatic choice by the units' CPML
+ * share, one detector, no exact reversal, and an unscaled tape format; else
  * FDTD_EINVAL.  fdtd_batch_backward needs the handles' forwards to come
  * from one fdtd_batch_forward (or with one record config). */
 int fdtd_batch_forward(fdtd_handle* const* hs, int n, const float* const* d_eps,
@@ -330,7 +332,8 @@ enum {
                                    automatic: small grids the direct half-steps (one pair of
                                    cells per thread; only with the default shape options),
                                    larger ones the split half-steps, from 12 million cells
-                                   on two steps per pass (3) where it can run (below), at
+                                   on (24 million with one z group by name) two steps per
+                                   pass (3) where it can run (below), at
                                    most half of the (tile, z chunk) units carrying CPML
                                    terms, else the fused step; 1 = split: an H and an E
                                    half-step launch, each updating the fields in place;

@@ -390,13 +390,14 @@ static void interp_weights(const fdtd_handle* h, const fdtd_record_cfg* rec, int
   }
 }
 
-// The reverse step of kernel 5 runs as two fused launches (primal and
-// adjoint, kernels_rev_fused.cu) unless FDTD_OPT_REVERSE asks for the split
-// phases; the fused kernels are built for 32 x 8 tiles.
-// Automatic (0): fused where at most half of the (tile, chunk) units carry
-// CPML terms, which its adjoint evaluates in a heavier variant (measured on
-// GB300: the reverse 11 % faster than split on 600 x 600 x 300 with 31 % of
-// the units in the CPML, 28 % slower on 200 x 200 x 100 with 70 %).
+// May the reverse step of kernel 5 run as the fused launches (the primal one and three
+// adjoint ones, kernels_rev_fused.cu)?  They are built for 32 x 8 tiles.  By name
+// (FDTD_OPT_REVERSE = 2) on any grid; automatic (0) where at most half of the (tile, chunk)
+// units carry CPML terms, which the adjoint evaluates in heavier variants, and the grid
+// is past the direct phases' line.  The half was drawn with earlier kernels; the present
+// ones beat the split phases beyond it too (us per reverse step, fused / split: 97 / 104 on
+// 200 x 200 x 100 with 70 % of the units in the CPML, 100 / 104 on 400 x 300 x 40), where the
+// workspace holds no second field and adjoint buffers.
 static bool fused_reverse(const fdtd_handle* h) {
   if (h->opt_kernel != 5 || h->opt_reverse == 1) return false;
   const int ty = h->opt_tile_y < 2 ? 2 : h->opt_tile_y;
@@ -427,14 +428,12 @@ static bool plane_meets(int axis, int index, int u0, int u1, int v0, int v1, con
          v1 > lo[va];
 }
 
-// The forward step of kernel 5 runs the units without a CPML term as one
-// fused launch (both half-steps, kernels_fwd_fused.cu) and the other units
-// with the split half-steps, unless FDTD_OPT_FORWARD asks for the split
-// half-steps everywhere.  It needs 32 x 8 tiles, such units, and the source
-// and the detector outside them (the split E half-step adds the source and
-// sums the objective).  Automatic (0): as the reverse step, fused where at
-// most half of the units carry CPML terms, unless the two-step pass (below)
-// runs there.
+// Is the fused forward step (kernels_fwd_fused.cu) one that a caller may name
+// (FDTD_OPT_FORWARD = 2), or that a named shape of the staged kernels takes by itself (at
+// most half of the units in the CPML)?  It needs 32 x 8 tiles, units without a CPML term,
+// and the source and the detector outside them: what the call has always asked for; the
+// kernels themselves take both in any unit, and the automatic choice on large grids
+// (forward_form) asks for none of it.
 static bool two_step_forward(const fdtd_handle* h);
 
 static bool fused_forward(const fdtd_handle* h) {
@@ -463,16 +462,13 @@ static bool fused_forward(const fdtd_handle* h) {
   return 2 * cpml <= all;
 }
 
-// Two time steps per pass (kernels_fwd_2step.cu, FDTD_OPT_FORWARD = 3): the
-// deep units run steps n and n + 1 in one launch, the other units the split
-// half-steps one step at a time through a third field buffer.  Needs kernel
-// 5 with 32 x 8 tiles, deep units, and the source and the detectors at least
-// two cells away from the deep box (the pass evaluates the intermediate
-// level on a two-cell halo and adds no source term, sums no objective).
-// Automatic (0): where the fused step would run (at most half of the units
-// carry CPML terms), which it beats on 600 x 600 x 300 (1028 against 1166 us
-// per forward step); on 200 x 200 x 100 it is slower than the split
-// half-steps (92 against 59 us), as the fused step is.
+// May two time steps run per pass (kernels_fwd_2step.cu, FDTD_OPT_FORWARD = 3)?  The deep
+// units run steps n and n + 1 in one launch, the other units the fused step one time step
+// at a time through a third field buffer.  Needs kernel 5 with 32 x 8 tiles, deep units,
+// and the source and the detectors at least two cells away from the deep box (the pass
+// evaluates the intermediate level on a two-cell halo and adds no source term, sums no
+// objective).  Automatic (0): at most half of the units in the CPML; from which size on it
+// is taken then: two_step_pays.
 static bool two_step_forward(const fdtd_handle* h) {
   if (h->opt_kernel != 5 || (h->opt_forward != 3 && h->opt_forward != 0)) return false;
   const int ty = h->opt_tile_y < 2 ? 2 : h->opt_tile_y;
@@ -551,11 +547,15 @@ static bool direct_reverse(const fdtd_handle* h) {
 // cache, where the fused launches' second buffers cost more than the second read
 // they save; beyond, two steps per pass where they may run (two_step_forward),
 // else the fused step, and the fused reverse step where it may (fused_reverse).  us
-// per step, forward split / fused / two steps: 60 / 73 / 85 on 200 x 200 x 100 (4 M
-// cells), 127 / 132 / 141 on 301 x 203 x 151 (9.2 M), 144 / 147 / 133 on 300 x 300 x
-// 120 (10.8 M), 176 / 175 / 153 on 300 x 300 x 150 (13.5 M), 406 / - / 315 on 411 x
-// 389 x 203 (32 M); reverse split / fused: 159 / 149 on 200 x 200 x 150 (6 M),
-// 196 / 178 on 260 x 200 x 150, 224 / 194 (9.2 M), 717 / 602 (32 M).  An
+// per step, forward split / fused / two steps: 60 / 73 / 88 on 200 x 200 x 100 (4 M
+// cells), 125 / 130 / 139 on 301 x 203 x 151 (9.2 M), 130 / - / 142 on 256 x 256 x 160
+// (10.5 M), 144 / 147 / 133 on 300 x 300 x 120 (10.8 M), 141 / - / 125 on 400 x 300 x 90 (10.8 M),
+// 151 / - / 134 on 340 x 340 x 100 (11.6 M), 176 / 175 / 153 on 300 x 300 x 150 (13.5 M), 406 / - /
+// 315 on 411 x 389 x 203 (32 M): the line by cells leaves 8 to 12 % on flat grids of 10 to
+// 12 M cells and keeps cubes below it from losing as much.  The fused step alone is even
+// with the split ones at 13.5 M (180 / 178 with the source in the deep box) and ahead from 15 M
+// on (185 / 196 on 500 x 500 x 60, 365 / 400 on 411 x 389 x 203).  Reverse split / fused: 151 / 138 on
+// 200 x 200 x 150 (6 M), 193 / 178 on 260 x 200 x 150, 225 / 195 (9.2 M), 717 / 602 (32 M).  An
 // option that names another shape of the split half-steps leaves the choice to the
 // units' CPML share alone.
 // With one z group (FDTD_OPT_ZGROUPS = 1) a pass and the other units' four launches
@@ -2158,7 +2158,7 @@ extern "C" int fdtd_value_and_grad_host(fdtd_handle* h, const float* h_eps,
 // L2 cache only while it stays there, so loops run side by side only as long as
 // their states fit into kGroupCacheShare of it together (one that does not fit by
 // itself counts as most of it and leaves room to small ones).  The plan is a list
-// schedule over estimated times, longest state first, smaller loops filling the room
+// schedule over estimated times, largest state first, smaller loops filling the room
 // left.  ms for twenty cubes of 48^3 to 128^3 / sixty-four of 32^3 to 128^3: 30.5 / 732
 // with 0.6 of the cache, 33.5 / 735 with 0.3, 31.6 / 691 with 1.0, 35.1 / 784 with 2, 35.5
 // / 811 all at once.

@@ -125,11 +125,12 @@ constexpr int adj_ctas() { return MODE == 2 ? 4 : (MODE == 1 ? 5 : 6); }
 // rows, each with all its chunks before the next group.  A chunk reads two planes
 // of its z neighbours: on a wide grid, taken layer by layer over the whole plane,
 // the neighbour's were read 100 MB and more ago and come from HBM again.  rows is
-// chosen (group_rows) so that a layer of a group is about one wave of resident
-// CTAs: smaller groups run several layers side by side, which costs more than it
-// saves.  us per reverse step on 600 x 600 x 300, 19 x 75 tiles: 1957 (75 rows, one
-// group), 1937 (60), 1922 (44), 1924 (38), 1936 (30), 1967 (15); on 411 x 389 x 203 (13
-// x 49, the one group that the rule takes) 616, in groups of 38 rows 623, of 25 630.
+// chosen (group_rows) for layers of about 750 units; smaller groups run several layers
+// side by side, which costs more than it saves.  The 750 is a measured figure (a wave of
+// either launch, six CTAs on each of 152 SMs, is 912).  us per reverse step on 600 x 600 x
+// 300, 19 x 75 tiles: 1957 (75 rows, one group), 1937 (60), 1922 (44), 1924 (38, the rule's
+// choice), 1936 (30), 1967 (15); on 411 x 389 x 203 (13 x 49, the one group that the rule
+// takes) 616, in groups of 38 rows 623, of 25 630.
 __device__ __forceinline__ int3 unit_order(int rows) {
   const unsigned gx = gridDim.x, gz = gridDim.z, u = blockIdx.x + gx * (blockIdx.y + gridDim.y * blockIdx.z);
   const unsigned per = gx * rows * gz, grp = u / per, r = u - grp * per;
@@ -138,8 +139,8 @@ __device__ __forceinline__ int3 unit_order(int rows) {
   return make_int3((int)(t - y * gx), (int)(grp * rows + y), (int)z);
 }
 inline int group_rows(dim3 grid) {
-  const unsigned wave = 750;   // five CTAs on each of 152 SMs
-  const unsigned n = (grid.x * grid.y + wave / 2) / wave;
+  const unsigned layer = 750;
+  const unsigned n = (grid.x * grid.y + layer / 2) / layer;
   return n > 1 ? (int)((grid.y + n - 1) / n) : (int)grid.y;
 }
 // Planes per chunk of a launch; zc: the chunk that the units are counted in.  Every
