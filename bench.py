@@ -618,9 +618,9 @@ def run_ours(args):
 # --------------------------------------------------------- profile run ---
 
 def run_profile(args):
-    """One short forward + backward with the given launch options, for profilers: the
-    launches one after another (one z group) unless --zgroups says otherwise or a
-    direction runs the direct half-steps, which one z group by name would replace."""
+    """One short forward + backward with the given launch options, for profilers: split
+    half-steps as one launch each (one z group) unless --zgroups says otherwise or the
+    other direction runs the direct ones, which one z group by name would replace."""
     import torch
     from paper_2603_24027_gb300 import _capi as A
     from paper_2603_24027_gb300 import build as B
@@ -634,7 +634,8 @@ def run_profile(args):
     rec = tape_cfg(A, args.tape)
     sim = fdtd.Simulation(w)
     apply_options(A, sim, args)
-    if args.zgroups == 0 and "direct" not in sim.step_forms().values():
+    forms = sim.step_forms().values()
+    if args.zgroups == 0 and "split" in forms and "direct" not in forms:
         sim.set_option(A.OPT_ZGROUPS, 1)
     sim.set_option(A.OPT_SAMPLE_EVERY, args.sample_every if args.sample_every != 50 else 0)
     eps = torch.from_numpy(w.eps).cuda()

@@ -1685,7 +1685,8 @@ static cudaError_t enqueue_backward(fdtd_handle* h, const fdtd_record_cfg* rec, 
   // sampled or one launch per half-step is asked for (FDTD_OPT_ZGROUPS = 1)
   const bool conc = fused && h->opt_sample == 0 && h->opt_zgroups != 1 && !h->one_stream &&
                     h->zs.size() >= 3 && h->zev.size() >= 9;
-  a.overlap = conc;
+  // sampled timing runs the launches in a row, but the same launches
+  a.overlap = h->opt_zgroups != 1 && !h->one_stream;
   for (int b = 0; fused && b < 2; ++b)
     if ((e = encode_rev_maps((const float*)(h->ws + L.F[b]), (const float*)(h->ws + L.L[b]),
                              (const float*)(h->ws + L.cb), (const float*)(h->ws + L.psiL[b]), a.g,

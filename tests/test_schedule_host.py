@@ -45,14 +45,16 @@ def ring_tiles(nx, ny, nz, P, zchunk):
     return -(-nx // 32) * -(-ny // 8) - box
 
 
+@pytest.mark.parametrize("sample", [0, 50])   # sampled runs time the same launches
 @pytest.mark.parametrize("grid,zgroups,zchunk,planes", [
     ((100, 100, 50, 8), 0, 8, 8), ((128, 128, 128, 8), 0, 8, 8), ((200, 200, 100, 12), 0, 8, 16),
     ((200, 200, 100, 12), 1, 8, 8), ((301, 203, 151, 10), 0, 8, 24), ((301, 203, 151, 10), 1, 8, 8),
     ((301, 203, 151, 10), 0, 4, 12), ((301, 203, 151, 10), 0, 16, 16), ((301, 203, 151, 10), 0, 0, 151)])
-def test_ring_chunks_grow_where_other_launches_hide_them(run, grid, zgroups, zchunk, planes):
+def test_ring_chunks_grow_where_other_launches_hide_them(run, grid, zgroups, zchunk, planes,
+                                                          sample):
     nx, ny, nz, P = grid
     sim = run.sim(problem(*grid), REC, {A.OPT_REVERSE: 2, A.OPT_ZGROUPS: zgroups,
-                                        A.OPT_ZCHUNK: zchunk})
+                                        A.OPT_ZCHUNK: zchunk, A.OPT_SAMPLE_EVERY: sample})
     run.forward(sim, REC)
     ring = [e.grid for e in run.backward(sim) if e.what == "launch" and "k_rev_adjoint" in e.name
             and e.grid[1:] == (1, 1)]
